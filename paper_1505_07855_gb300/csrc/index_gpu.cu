@@ -6,10 +6,9 @@
 //
 // Suffix array by prefix doubling (Manber and Myers 1993, restricted to the
 // groups not yet sorted as in Larsson and Sadakane 2007):
-//   round 0: every suffix is keyed by its first 21 symbols (3 bits each, a real
-//            symbol c as c+1, past the end 0) and the (key, start) pairs are
-//            radix-sorted; equal keys form groups, and a suffix's rank is the
-//            row of its group's first member;
+//   round 0: every suffix is keyed by its first 16 symbols (24 for a long text)
+//            and the (key, start) pairs are radix-sorted; equal keys form groups,
+//            and a suffix's rank is the row of its group's first member;
 //   round h: the members of groups with two or more suffixes are keyed by
 //            (rank of the suffix, rank of the suffix h positions later), sorted,
 //            and split where the key changes; ranks are updated after every key
@@ -18,7 +17,7 @@
 // and rank[n] (the suffix "$") is 0.
 //
 // Device primitives written for this file: a tiled scan (sum or max) and an LSD
-// radix sort of (u64 key, u32 value) pairs, 8-bit digits, 4096-element tiles,
+// radix sort of (u32 or u64 key, u32 value) pairs, 8-bit digits, 4096-element tiles,
 // stable ranking inside a tile by warp match + per-warp digit counters, and a
 // shared-memory staging pass so that each digit's run is written contiguously.
 #include <cuda_runtime.h>
@@ -28,6 +27,7 @@
 #include <string>
 #include <vector>
 
+#include "aln_device.cuh"
 #include "aln_internal.h"
 #include "aln_scan.cuh"
 
@@ -47,9 +47,11 @@ constexpr int kRsWarps = kRsThreads / 32;
 constexpr int kRsRounds = 16;                                   // rounds of 32 items per warp
 constexpr uint32_t kRsTile = kRsThreads * kRsRounds;            // 4096 items per tile
 constexpr int kRsBins = 256;
-constexpr size_t kRsSmem = (kRsWarps * kRsBins + 2 * kRsBins) * 4 + kRsTile * (8 + 4);
+template <class K>
+constexpr size_t kRsSmem = (kRsWarps * kRsBins + 2 * kRsBins) * 4 + kRsTile * (sizeof(K) + 4);
 
-__global__ void __launch_bounds__(kRsThreads) rs_hist_kernel(const uint64_t *keys, uint64_t n, uint32_t shift,
+template <class K>
+__global__ void __launch_bounds__(kRsThreads) rs_hist_kernel(const K *keys, uint64_t n, uint32_t shift,
                                                              uint32_t *counts, uint64_t n_tiles) {
     __shared__ uint32_t h[kRsBins];
     h[threadIdx.x] = 0;
@@ -66,12 +68,13 @@ __global__ void __launch_bounds__(kRsThreads) rs_hist_kernel(const uint64_t *key
 
 // Stable scatter of one tile by the digit at `shift`.  offs: exclusive scan of
 // the digit-major counts (global start of digit d's part of tile t).
-__global__ void __launch_bounds__(kRsThreads) rs_scatter_kernel(const uint64_t *kin, const uint32_t *vin,
-                                                                uint64_t *kout, uint32_t *vout, uint64_t n,
+template <class K>
+__global__ void __launch_bounds__(kRsThreads) rs_scatter_kernel(const K *kin, const uint32_t *vin,
+                                                                K *kout, uint32_t *vout, uint64_t n,
                                                                 uint32_t shift, const uint32_t *offs,
                                                                 uint64_t n_tiles) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    uint64_t *sk = reinterpret_cast<uint64_t *>(smem_raw);
+    K *sk = reinterpret_cast<K *>(smem_raw);
     uint32_t *sv = reinterpret_cast<uint32_t *>(sk + kRsTile);
     uint32_t *whist = sv + kRsTile;            // [warp][digit]: running count, then offset in the tile's digit
     uint32_t *tdig = whist + kRsWarps * kRsBins;  // local start of each digit in the tile
@@ -81,14 +84,14 @@ __global__ void __launch_bounds__(kRsThreads) rs_scatter_kernel(const uint64_t *
     __syncthreads();
     const uint64_t base = static_cast<uint64_t>(blockIdx.x) * kRsTile;
     const uint32_t lt = (1u << lane) - 1u;
-    uint64_t k[kRsRounds];
+    K k[kRsRounds];
     uint32_t v[kRsRounds], pos[kRsRounds];
     uint32_t *wh = whist + warp * kRsBins;
 #pragma unroll
     for (int r = 0; r < kRsRounds; r++) {
         const uint64_t j = base + static_cast<uint64_t>(warp) * (32 * kRsRounds) + 32u * r + lane;
         const bool valid = j < n;
-        k[r] = valid ? kin[j] : 0ull;
+        k[r] = valid ? kin[j] : K(0);
         v[r] = valid ? vin[j] : 0u;
         const uint32_t d = valid ? static_cast<uint32_t>((k[r] >> shift) & 255u) : 256u;
         const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
@@ -128,7 +131,7 @@ __global__ void __launch_bounds__(kRsThreads) rs_scatter_kernel(const uint64_t *
     for (int i = 0; i < kRsRounds; i++) {
         const uint32_t t = i * kRsThreads + threadIdx.x;
         if (t < cnt) {
-            const uint64_t key = sk[t];
+            const K key = sk[t];
             const uint32_t d = static_cast<uint32_t>((key >> shift) & 255u);
             const uint64_t g = static_cast<uint64_t>(offs[static_cast<uint64_t>(d) * n_tiles + blockIdx.x]) + (t - tdig[d]);
             kout[g] = key;
@@ -138,7 +141,7 @@ __global__ void __launch_bounds__(kRsThreads) rs_scatter_kernel(const uint64_t *
 }
 
 struct SortBufs {
-    uint64_t *k[2];
+    uint64_t *k[2];    // keys of up to 64 bits (a sort of 32-bit keys uses half of each)
     uint32_t *v[2];
     uint32_t *counts;  // kRsBins * tiles
     uint32_t *scan_tmp;
@@ -146,15 +149,17 @@ struct SortBufs {
 
 // Sort n pairs in (k[0], v[0]) by the low `bits` bits of the key (stable LSD);
 // returns the index (0 or 1) of the buffers holding the result.
+template <class K>
 int radix_sort(SortBufs &B, uint64_t n, uint32_t bits, cudaStream_t st) {
     int cur = 0;
     if (n <= 1) return cur;
+    K *key[2] = {reinterpret_cast<K *>(B.k[0]), reinterpret_cast<K *>(B.k[1])};
     const uint64_t tiles = (n + kRsTile - 1) / kRsTile;
     for (uint32_t shift = 0; shift < bits; shift += 8) {
-        rs_hist_kernel<<<static_cast<unsigned>(tiles), kRsThreads, 0, st>>>(B.k[cur], n, shift, B.counts, tiles);
+        rs_hist_kernel<K><<<static_cast<unsigned>(tiles), kRsThreads, 0, st>>>(key[cur], n, shift, B.counts, tiles);
         device_scan(B.counts, B.counts, kRsBins * tiles, false, B.scan_tmp, st, OpAdd());
-        rs_scatter_kernel<<<static_cast<unsigned>(tiles), kRsThreads, kRsSmem, st>>>(
-            B.k[cur], B.v[cur], B.k[cur ^ 1], B.v[cur ^ 1], n, shift, B.counts, tiles);
+        rs_scatter_kernel<K><<<static_cast<unsigned>(tiles), kRsThreads, kRsSmem<K>, st>>>(
+            key[cur], B.v[cur], key[cur ^ 1], B.v[cur ^ 1], n, shift, B.counts, tiles);
         cur ^= 1;
     }
     return cur;
@@ -181,27 +186,45 @@ __global__ void text_kernel(const uint8_t *text, uint64_t n, uint64_t seed, uint
     }
 }
 
-// Round 0 keys: suffix i (0..n) keyed by its first 21 symbols.
-__global__ void key21_kernel(const uint8_t *y, uint64_t n, uint64_t *key, uint32_t *val) {
-    const uint64_t N = n + 1;
-    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < N;
-         i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        uint64_t k = 0;
+// 16 symbols in 32 bits take 4 sort passes of 8-byte pairs, where 21 symbols of 3
+// bits took 8 passes of 12-byte pairs; a text of 100 Mbp leaves a few per cent of
+// its suffixes to the later rounds (build and upload 79 -> 65 ms with the table
+// below; the passes are bound by the scattered stores of the digits' runs).
+//
+// Round 0 keys: the suffixes from the last (n, "$") to the first, keyed by their
+// first kFirst<K> symbols, 2 bits each, past the end as A.  A suffix of fewer
+// symbols sorts before the longer ones of the same key: the sort is stable, and
+// of two suffixes the later one, which comes first here, is the shorter one.
+template <class K>
+constexpr uint32_t kFirst = sizeof(K) == 4 ? 16 : 24;
+
+template <class K>
+__global__ void first_key_kernel(const uint8_t *y, uint64_t n, K *key, uint32_t *val) {
+    for (uint64_t t = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; t <= n;
+         t += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
+        const uint64_t i = n - t;
+        K k = 0;
 #pragma unroll
-        for (int t = 0; t < 21; t++) {
-            const uint64_t p = i + t;
-            k = (k << 3) | (p < n ? static_cast<uint64_t>(y[p]) + 1u : 0u);
-        }
-        key[i] = k;
-        val[i] = static_cast<uint32_t>(i);
+        for (uint32_t u = 0; u < kFirst<K>; u++) k = (k << 2) | (i + u < n ? K(y[i + u]) : K(0));
+        key[t] = k;
+        val[t] = static_cast<uint32_t>(i);
     }
 }
 
+// Whether sorted row i starts a run of suffixes not told apart yet: its key is
+// another one, or the suffix before it has fewer symbols than the key (val is
+// given in round 0, when n - val can be below `first`).
+template <class K>
+__device__ __forceinline__ bool run_starts(const K *key, const uint32_t *val, uint64_t n, uint32_t first, uint64_t i) {
+    return i == 0 || key[i] != key[i - 1] || (val && n - val[i - 1] < first);
+}
+
 // head[i] = i where key[i] starts a run of equal keys, else 0 (max-scan input).
-__global__ void run_head_kernel(const uint64_t *key, uint64_t m, uint32_t *head) {
+template <class K>
+__global__ void run_head_kernel(const K *key, const uint32_t *val, uint64_t n, uint64_t m, uint32_t *head) {
     for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < m;
          i += static_cast<uint64_t>(gridDim.x) * blockDim.x)
-        head[i] = (i == 0 || key[i] != key[i - 1]) ? static_cast<uint32_t>(i) : 0u;
+        head[i] = run_starts(key, val, n, kFirst<K>, i) ? static_cast<uint32_t>(i) : 0u;
 }
 
 // After a sort of the active rows: the suffix order goes back into sa at the
@@ -219,23 +242,25 @@ __global__ void place_rank_kernel(const uint32_t *A, const uint32_t *v, const ui
 }
 
 // active[i] = 1 if row i's run has two or more members (keys sorted).
-__global__ void active_kernel(const uint64_t *key, uint64_t m, uint32_t *active) {
+template <class K>
+__global__ void active_kernel(const K *key, const uint32_t *val, uint64_t n, uint64_t m, uint32_t *active) {
     for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < m;
          i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        const bool head = i == 0 || key[i] != key[i - 1];
-        const bool next_head = i + 1 == m || key[i + 1] != key[i];
+        const bool head = run_starts(key, val, n, kFirst<K>, i);
+        const bool next_head = i + 1 == m || run_starts(key, val, n, kFirst<K>, i + 1);
         active[i] = (head && next_head) ? 0u : 1u;
     }
 }
 
 // Compaction: rows of active runs, in order.  pos = inclusive scan of the
 // flags; flags are recomputed from the keys (the flag array was scanned in place).
-__global__ void compact_kernel(const uint64_t *key, const uint32_t *A, const uint32_t *pos, uint64_t m,
-                               uint32_t *A2) {
+template <class K>
+__global__ void compact_kernel(const K *key, const uint32_t *val, uint64_t n, const uint32_t *A, const uint32_t *pos,
+                               uint64_t m, uint32_t *A2) {
     for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < m;
          i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        const bool head = i == 0 || key[i] != key[i - 1];
-        const bool next_head = i + 1 == m || key[i + 1] != key[i];
+        const bool head = run_starts(key, val, n, kFirst<K>, i);
+        const bool next_head = i + 1 == m || run_starts(key, val, n, kFirst<K>, i + 1);
         if (!(head && next_head)) A2[pos[i] - 1] = A ? A[i] : static_cast<uint32_t>(i);
     }
 }
@@ -343,38 +368,23 @@ __global__ void primary_count_kernel(const uint32_t *sa, const uint8_t *y, uint6
     if (threadIdx.x < 4) atomicAdd(&cnt[threadIdx.x], c[threadIdx.x]);
 }
 
-// The first min(k, n - s) symbols of the suffix at row r as a base-4 number,
-// first symbol lowest (the order the search processes them), with the count of
-// available symbols in bits 24..27.
-__global__ void kmer_id_kernel(const uint8_t *y, const uint32_t *sa, uint64_t n, uint32_t k, uint32_t *id) {
-    for (uint64_t r = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; r <= n;
-         r += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        const uint64_t s = sa[r];
-        const uint32_t avail = static_cast<uint32_t>(n - s < k ? n - s : k);
-        uint32_t v = 0;
-        for (uint32_t u = 0; u < avail; u++) v |= static_cast<uint32_t>(y[s + u]) << (2 * u);
-        id[r] = v | (avail << 24);
+// Prefix-trie table, one level a launch: the intervals of the four extensions of
+// every string of length j (absent strings are (0, 0), and so are theirs).  A
+// level takes one pair of Occ reads a string, where a pass over the rows would
+// read the text at every suffix (3.1 Gbp, depth 10: 0.16 s a text; now 50 us).
+__global__ void kmer_level_kernel(DText T, uint32_t strings, const uint2 *level, uint4 *next) {
+    const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= strings) return;
+    const uint2 iv = level ? level[s] : make_uint2(0u, T.n + 1u);
+    uint32_t lo[4] = {0, 0, 0, 0}, hi[4] = {0, 0, 0, 0};
+    if (iv.y > iv.x) {
+        lf4(T, iv.x, iv.y, lo, hi);
+#pragma unroll
+        for (int c = 0; c < 4; c++)
+            if (hi[c] <= lo[c]) lo[c] = hi[c] = 0;
     }
-}
-
-// Prefix-trie table: for every level j, the run of rows whose j-prefix is the
-// string with index i sets entry (lo, hi) = (first row, last row + 1).
-__global__ void kmer_table_kernel(const uint32_t *id, uint64_t N, uint32_t k, uint32_t *kmer) {
-    for (uint64_t r = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; r < N;
-         r += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        const uint32_t cur = id[r];
-        const uint32_t prv = r > 0 ? id[r - 1] : 0u, nxt = r + 1 < N ? id[r + 1] : 0u;
-        for (uint32_t j = 1; j <= k; j++) {
-            if ((cur >> 24) < j) break;
-            const uint32_t mask = (1u << (2 * j)) - 1u;
-            const uint32_t me = cur & mask;
-            const uint64_t off = ((1ull << (2 * j)) - 4) / 3 + me;
-            const bool first = r == 0 || (prv >> 24) < j || (prv & mask) != me;
-            const bool last = r + 1 == N || (nxt >> 24) < j || (nxt & mask) != me;
-            if (first) kmer[2 * off] = static_cast<uint32_t>(r);
-            if (last) kmer[2 * off + 1] = static_cast<uint32_t>(r + 1);
-        }
-    }
+    next[2 * s] = make_uint4(lo[0], hi[0], lo[1], hi[1]);
+    next[2 * s + 1] = make_uint4(lo[2], hi[2], lo[3], hi[3]);
 }
 
 unsigned grid_for(uint64_t n, int threads) {
@@ -403,42 +413,65 @@ struct DevMem {
 
 }  // namespace
 
+// After a sort of the m active rows by key: their suffixes' places and ranks, and
+// the rows of the runs that are left (*left of them) in Anext.
+template <class K>
+static cudaError_t place_round(const SortBufs &B, int c, const uint32_t *val, uint64_t n, uint64_t m,
+                               const uint32_t *Acur, uint32_t *Anext, uint32_t *sa, uint32_t *rank, uint32_t *tmp,
+                               uint32_t *left, cudaStream_t st) {
+    const int T = 256;
+    const K *key = reinterpret_cast<const K *>(B.k[c]);
+    // ranks: the row of the first member of each run of equal keys
+    run_head_kernel<K><<<grid_for(m, T), T, 0, st>>>(key, val, n, m, tmp);
+    device_scan(tmp, tmp, m, true, B.scan_tmp, st, OpMax());
+    place_rank_kernel<<<grid_for(m, T), T, 0, st>>>(Acur, B.v[c], tmp, m, sa, rank);
+    // rows of runs with two or more members stay active
+    active_kernel<K><<<grid_for(m, T), T, 0, st>>>(key, val, n, m, tmp);
+    device_scan(tmp, tmp, m, true, B.scan_tmp, st, OpAdd());
+    compact_kernel<K><<<grid_for(m, T), T, 0, st>>>(key, val, n, Acur, tmp, m, Anext);
+    const cudaError_t e = cudaMemcpyAsync(left, tmp + (m - 1), 4, cudaMemcpyDeviceToHost, st);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+}
+
+// Round 0: every suffix by its first kFirst<K> symbols.
+template <class K>
+static cudaError_t first_round(const uint8_t *y, uint64_t n, uint32_t *sa, uint32_t *rank, uint32_t *A, uint32_t *tmp,
+                               SortBufs &B, uint32_t *left, cudaStream_t st) {
+    const uint64_t N = n + 1;
+    first_key_kernel<K><<<grid_for(N, 256), 256, 0, st>>>(y, n, reinterpret_cast<K *>(B.k[0]), B.v[0]);
+    const int c = radix_sort<K>(B, N, 2 * kFirst<K>, st);
+    return place_round<K>(B, c, B.v[c], n, N, nullptr, A, sa, rank, tmp, left, st);
+}
+
+// Texts from which round 0 takes the longer keys: 4^16 strings leave about half
+// the suffixes of a random text of 3 Gbp in groups, 4^24 next to none.
+constexpr uint64_t kLongKeys = 1ull << 29;
+
 // Suffix array of y$ (y on the device, codes 0..3, length n) into sa (n + 1 rows).
 // rank, A, A2, tmp: n + 1 words each.
 static cudaError_t gpu_suffix_array(const uint8_t *y, uint64_t n, uint32_t *sa, uint32_t *rank, uint32_t *A,
                                     uint32_t *A2, uint32_t *tmp, SortBufs &B, cudaStream_t st) {
     const uint64_t N = n + 1;
-    const int T = 256;
-    cudaError_t e;
-    key21_kernel<<<grid_for(N, T), T, 0, st>>>(y, n, B.k[0], B.v[0]);
-    int c = radix_sort(B, N, 63, st);
-    uint64_t m = N;
-    const uint32_t *Acur = nullptr;  // round 0: the active rows are all rows
+    const bool wide = n >= kLongKeys;
+    uint32_t left = 0;
+    cudaError_t e = wide ? first_round<uint64_t>(y, n, sa, rank, A, tmp, B, &left, st)
+                         : first_round<uint32_t>(y, n, sa, rank, A, tmp, B, &left, st);
     uint32_t b = 1;
     while (b < 32 && (1ull << b) < N) b++;
-    uint64_t h = 21;
-    for (int round = 0;; round++) {
-        // ranks: the row of the first member of each run of equal keys
-        run_head_kernel<<<grid_for(m, T), T, 0, st>>>(B.k[c], m, tmp);
-        device_scan(tmp, tmp, m, true, B.scan_tmp, st, OpMax());
-        place_rank_kernel<<<grid_for(m, T), T, 0, st>>>(Acur, B.v[c], tmp, m, sa, rank);
-        // rows of runs with two or more members stay active
-        active_kernel<<<grid_for(m, T), T, 0, st>>>(B.k[c], m, tmp);
-        device_scan(tmp, tmp, m, true, B.scan_tmp, st, OpAdd());
-        uint32_t *Anext = (Acur == A) ? A2 : A;
-        compact_kernel<<<grid_for(m, T), T, 0, st>>>(B.k[c], Acur, tmp, m, Anext);
-        uint32_t m2 = 0;
-        if ((e = cudaMemcpyAsync(&m2, tmp + (m - 1), 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-        if (m2 == 0) break;
+    uint64_t h = wide ? kFirst<uint64_t> : kFirst<uint32_t>;
+    uint32_t *Acur = A, *Anext = A2;
+    for (int round = 0; e == cudaSuccess && left; round++) {
         if (round >= 34 || h > 2 * N) return cudaErrorUnknown;  // cannot happen: runs share h real symbols
+        const uint64_t m = left;
+        round_key_kernel<<<grid_for(m, 256), 256, 0, st>>>(Acur, m, sa, rank, h, n, b, B.k[0], B.v[0]);
+        const int c = radix_sort<uint64_t>(B, m, 2 * b, st);
+        e = place_round<uint64_t>(B, c, nullptr, n, m, Acur, Anext, sa, rank, tmp, &left, st);
+        uint32_t *t = Acur;
         Acur = Anext;
-        m = m2;
-        round_key_kernel<<<grid_for(m, T), T, 0, st>>>(Acur, m, sa, rank, h, n, b, B.k[0], B.v[0]);
-        c = radix_sort(B, m, 2 * b, st);
+        Anext = t;
         h *= 2;
     }
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace aln
@@ -498,8 +531,10 @@ extern "C" int fm_index_build_gpu(const uint8_t *text, uint64_t n, const fm_buil
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             if (d_text) cudaFree(d_text);
         }
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(rs_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       static_cast<int>(kRsSmem));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(rs_scatter_kernel<uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       static_cast<int>(kRsSmem<uint64_t>));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(rs_scatter_kernel<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       static_cast<int>(kRsSmem<uint32_t>));
         if (e == cudaSuccess) {
             try {
                 ix = new fm_index();
@@ -522,14 +557,30 @@ extern "C" int fm_index_build_gpu(const uint8_t *text, uint64_t n, const fm_buil
             cudaMemsetAsync(misc, 0, 8 * sizeof(unsigned long long), st);
             primary_count_kernel<<<grid_for(N, 256) < 4096 ? grid_for(N, 256) : 4096, 256, 0, st>>>(sa, y, n, misc,
                                                                                                   misc + 1);
-            if (o.kmer_k) {
-                kmer_id_kernel<<<grid_for(N, 256), 256, 0, st>>>(y, sa, n, o.kmer_k, tmp);
-                cudaMemsetAsync(kmer, 0, kwords * 4, st);
-                kmer_table_kernel<<<grid_for(N, 256), 256, 0, st>>>(tmp, N, o.kmer_k, kmer);
-            }
-            if ((e = cudaGetLastError()) != cudaSuccess) break;
             HostText &Tt = ix->t[w];
             unsigned long long hm[5];
+            if ((e = cudaMemcpyAsync(hm, misc, sizeof hm, cudaMemcpyDeviceToHost, st)) != cudaSuccess) break;
+            if ((e = cudaStreamSynchronize(st)) != cudaSuccess) break;
+            Tt.n = n;
+            Tt.primary = hm[0];
+            Tt.C[0] = 0;
+            for (int cc = 1; cc < 4; cc++) Tt.C[cc] = Tt.C[cc - 1] + hm[cc];
+            DText D{};
+            D.blocks = reinterpret_cast<const uint4 *>(blocks);
+            for (int cc = 0; cc < 4; cc++) D.C1[cc] = static_cast<uint32_t>(Tt.C[cc] + 1);
+            D.C1[4] = static_cast<uint32_t>(n + 1);
+            D.primary = static_cast<uint32_t>(Tt.primary);
+            D.n = static_cast<uint32_t>(n);
+            const uint2 *level = nullptr;
+            uint2 *next = reinterpret_cast<uint2 *>(kmer);
+            for (uint32_t j = 0; j < o.kmer_k; j++) {
+                const uint32_t strings = 1u << (2 * j);
+                kmer_level_kernel<<<(strings + 255u) / 256u, 256, 0, st>>>(D, strings, level,
+                                                                          reinterpret_cast<uint4 *>(next));
+                level = next;
+                next += 4ull * strings;
+            }
+            if ((e = cudaGetLastError()) != cudaSuccess) break;
             try {
                 Tt.blocks.resize(nb * 16);
                 Tt.sa_samp.resize(ns);
@@ -542,13 +593,7 @@ extern "C" int fm_index_build_gpu(const uint8_t *text, uint64_t n, const fm_buil
             if ((e = cudaMemcpyAsync(Tt.sa_samp.data(), samp, ns * 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess) break;
             if (kwords && (e = cudaMemcpyAsync(Tt.kmer.data(), kmer, kwords * 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
                 break;
-            if ((e = cudaMemcpyAsync(hm, misc, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
-                break;
             if ((e = cudaStreamSynchronize(st)) != cudaSuccess) break;
-            Tt.n = n;
-            Tt.primary = hm[0];
-            Tt.C[0] = 0;
-            for (int cc = 1; cc < 4; cc++) Tt.C[cc] = Tt.C[cc - 1] + hm[cc];
         }
         if (rc == ALN_OK && e != cudaSuccess)
             rc = fail(e == cudaErrorMemoryAllocation ? ALN_ENOMEM : ALN_EDEVICE,
