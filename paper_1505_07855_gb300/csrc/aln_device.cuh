@@ -35,6 +35,7 @@ struct DIndex {
     DText t[2];              // t[0] = X, t[1] = X reversed
     uint32_t kmer_k;
     uint32_t sa_shift;       // log2(sa_sample)
+    const uint32_t *sa[2];   // every SA value of X and of X reversed (derived at upload), or nullptr
 };
 
 __device__ __forceinline__ uint4 ld_nc(const uint4 *p) {
