@@ -146,8 +146,13 @@ int fm_index_load(const char *path, fm_index **out);
  * memory).  device: CUDA ordinal.  The copy is enqueued on stream and finished
  * before return.  The library allocates the device image (Occ blocks, sampled SA
  * and k-mer table of both texts) and a stream-ordered memory pool for the
- * search's per-call scratch; ALN_ENOMEM if it does not fit.  Free with
- * fm_dindex_free. */
+ * search's per-call scratch; ALN_ENOMEM if it does not fit.  Where they take at
+ * most a quarter of the device memory that is then free, it also derives from the
+ * image the whole suffix array of both texts, its inverse at every fourth
+ * position, the text as bit planes and, for every string of up to 16 bases, the
+ * number of suffixes below it (14 to 26 bytes a base in all): the search and
+ * sa_to_pos give the same results with or without them, and are faster with them.
+ * Free with fm_dindex_free. */
 int fm_index_to_device(const fm_index *idx, int device, void *stream, fm_dindex **out);
 void fm_dindex_free(fm_dindex *d);
 int fm_dindex_info(const fm_dindex *d, fm_index_info_t *info);
@@ -195,7 +200,9 @@ typedef struct {
                                process's persisting-L2 set-aside (cudaLimitPersistingL2CacheSize,
                                a limit of the CUDA context) to the window size; 0 = off;
                                result-neutral */
-    uint32_t work_limit;    /* node expansions per read before ALN_FLAG_WORK_LIMIT; 0 = 2^24 */
+    uint32_t work_limit;    /* node expansions per read before ALN_FLAG_WORK_LIMIT; 0 = 2^24;
+                               with this or loop_limit set, every read goes to the tree search
+                               that they bound (see aln_search) */
     uint32_t loop_limit;    /* persistent form: trips of the kernel's loop per warp before the
                                warp stops (ALN_STATUS_LOOP_LIMIT, unfinished reads flagged
                                ALN_FLAG_LOOP_LIMIT); 0 = 64 * n_reads * (576 + work_limit),
@@ -280,7 +287,13 @@ typedef struct {
  * its unfinished reads ALN_FLAG_LOOP_LIMIT and flags every read it then takes
  * from the queue the same way without searching it, so every read gets a
  * result; the binding turns the status bit into ALN_ELIMIT.
- * Persistent mode first computes every read's D array in a pre-pass and visits
+ * With the derived arrays (fm_index_to_device), at most one gap open in reach
+ * (max_gapo or z at most 1) and neither work_limit nor loop_limit set, both forms
+ * first answer each read from the places of its error-free parts (a transcript
+ * with b differences leaves one of b + 1 parts of the read as it is); the reads
+ * with too many places or targets for that go to the tree search.  In persistent
+ * mode this needs a scratch, as below.
+ * Persistent mode else first computes every read's D array in a pre-pass and visits
  * reads in decreasing order of their lower bound; in the batch's tail (the
  * read queue empty) reads past params.heavy_after expansions of their owner
  * lane are handed to the heavy phase (at most 2048 per call), which searches

@@ -70,6 +70,7 @@ static int search_params(const char *who, const aln_params &P, uint32_t n_reads,
     sp.sc_go = P.score_gapo ? P.score_gapo : 11;
     sp.sc_ge = P.score_gape ? P.score_gape : 4;
     sp.max_best = P.max_best;
+    sp.bounded = P.work_limit || P.loop_limit;
     sp.heavy.hdr = nullptr;
     if (P.l2_window > 1) return fail(ALN_EINVAL, std::string(who) + ": l2_window must be 0 or 1");
     sp.window_base = nullptr;

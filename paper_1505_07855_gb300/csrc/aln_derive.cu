@@ -1,13 +1,17 @@
 // Arrays derived on the device from the uploaded index: the whole suffix array
-// of both texts (the index keeps every sa_sample-th row).  They follow from the
-// image alone, so a search or a position look-up gives the same numbers with or
-// without them; an index whose arrays would not fit comfortably is served from
-// the image.
+// of both texts (the index keeps every sa_sample-th row), its inverse at every
+// kIsaStep-th text position, the text X as bit planes, and for every string of
+// lo_k bases the number of suffixes of X below it.  They follow from the image
+// alone, so a search or a position look-up gives the same numbers with or without
+// them; an index whose arrays would not fit comfortably is served from the image.
 //
-// The suffix array comes from LF walks: from the sampled row r, whose value is
-// known, LF leads to the row of the suffix one position earlier, until the next
-// sampled row.  Every row lies on exactly one such walk, so the n + 1 rows take
-// n LF steps in all, one thread per sampled row.
+// The first three come from LF walks: from the sampled row r, whose value is
+// known, LF leads to the row of the suffix one position earlier, and shows the
+// base there, until the next sampled row.  Every row lies on exactly one such
+// walk, so the n + 1 rows take n LF steps in all, one thread per sampled row.
+// The table follows from the Occ counts, one base longer a launch: the suffixes
+// below c s are those that start with a lower base and those of base c whose
+// rest is below s.
 #include <cuda_runtime.h>
 
 #include "aln_device.cuh"
@@ -16,6 +20,11 @@
 namespace aln {
 namespace {
 
+__device__ __forceinline__ void put_bases(uint2 *text, uint32_t word, uint32_t lo, uint32_t hi) {
+    if (lo) atomicOr(&text[word].x, lo);
+    if (hi) atomicOr(&text[word].y, hi);
+}
+
 constexpr uint32_t kWalkError = 1u;   // a walk left the text, missed its sample or passed its bound
 
 // One thread per sampled row: the walk to the next sampled row.  Bound by the
@@ -23,14 +32,16 @@ constexpr uint32_t kWalkError = 1u;   // a walk left the text, missed its sample
 // stores); one thread per walk keeps the most walks in flight.  Both texts of
 // 100 Mbp add about 8 ms to the upload.
 __global__ void __launch_bounds__(256) sa_fill_kernel(DText T, uint32_t shift, uint32_t limit, uint32_t n_samples,
-                                                      uint32_t *sa, uint32_t *err) {
+                                                      uint32_t *sa, uint32_t *isa, uint2 *text, uint32_t *err) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_samples) return;
     const uint32_t mask = (1u << shift) - 1u;
     uint32_t row = i << shift, v = T.sa_samp[i], steps = 0;
     bool bad = v > T.n;
+    uint32_t lo = 0, hi = 0, word = v >> 5;  // bases of the text word the walk is in
     while (!bad) {
         sa[row] = v;
+        if (v % kIsaStep == 0) isa[v / kIsaStep] = row;
         if (row == T.primary) {  // SA[primary] = 0: the walk around the text ends here
             bad = v != 0;
             break;
@@ -39,9 +50,19 @@ __global__ void __launch_bounds__(256) sa_fill_kernel(DText T, uint32_t shift, u
             bad = true;
             break;
         }
-        row = lf_row(T, row);
+        uint32_t c;
+        row = lf_row(T, row, c);
         v--;
         steps++;
+        if (text) {
+            if (v >> 5 != word) {
+                put_bases(text, word, lo, hi);
+                lo = hi = 0;
+                word = v >> 5;
+            }
+            lo |= (c & 1u) << (v & 31u);
+            hi |= (c >> 1) << (v & 31u);
+        }
         if (row > T.n) {
             bad = true;
         } else if ((row & mask) == 0) {
@@ -49,12 +70,45 @@ __global__ void __launch_bounds__(256) sa_fill_kernel(DText T, uint32_t shift, u
             break;
         }
     }
+    if (text && !bad) put_bases(text, word, lo, hi);
     if (bad) atomicOr(err, kWalkError);
+}
+
+// lo[c 4^j + s] = number of suffixes below the string c s, from lo[s] over the
+// 4^j strings s (first base highest), in place: a thread reads entry s alone and
+// writes that entry and three past the level.
+__global__ void __launch_bounds__(256) lo_level_kernel(DText T, uint64_t strings, uint32_t *lo) {
+    const uint64_t s = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (s >= strings) return;
+    const uint32_t at = lo[s];
+    const uint32_t b = at / kRowsPerBlock, o = at - b * kRowsPerBlock;
+    HalfBlock H;
+    load_half(T.blocks, b, o, H);
+    uint32_t occ[4];
+    occ4_in_half(H, o, occ);
+    occ[0] -= at > T.primary ? 1u : 0u;
+#pragma unroll
+    for (int c = 0; c < 4; c++) lo[c * strings + s] = T.C1[c] + occ[c];
 }
 
 }  // namespace
 
-uint64_t derived_bytes(uint64_t n) { return 256 + 2 * derived_align(4 * (n + 1)); }
+static uint64_t text_words(uint64_t n) { return n / 32 + 1 + 2 * kTextPad; }
+
+// Depth of the table: the strings number at most kLoStrings times the suffixes,
+// so that a random string of that length is met less than once.
+static uint32_t lo_depth(uint64_t n) {
+    uint32_t k = 1;
+    while (k < 16 && (4ull << (2 * k)) <= kLoStrings * (n + 1)) k++;
+    return k;
+}
+
+static uint64_t lo_entries(uint64_t n) { return (1ull << (2 * lo_depth(n))) + 1; }
+
+uint64_t derived_bytes(uint64_t n) {
+    return 256 + 2 * derived_align(4 * (n + 1)) + 2 * derived_align(4 * (n / kIsaStep + 1)) +
+           derived_align(8 * text_words(n)) + derived_align(4 * lo_entries(n));
+}
 
 // The derived arrays of index X in mem (derived_bytes(n) bytes), on stream st;
 // *ok tells whether the image was consistent (walks that met their samples
@@ -62,26 +116,44 @@ uint64_t derived_bytes(uint64_t n) { return 256 + 2 * derived_align(4 * (n + 1))
 cudaError_t derive(DIndex &X, void *mem, cudaStream_t st, bool *ok) {
     const uint64_t n = X.t[0].n;
     char *p = static_cast<char *>(mem);
-    uint32_t *err = reinterpret_cast<uint32_t *>(p);
-    p += 256;
+    auto take = [&](uint64_t bytes) {
+        char *at = p;
+        p += derived_align(bytes);
+        return at;
+    };
     *ok = false;
+    uint32_t *err = reinterpret_cast<uint32_t *>(take(256));
+    uint32_t *sa[2], *isa[2];
+    for (int w = 0; w < 2; w++) sa[w] = reinterpret_cast<uint32_t *>(take(4 * (n + 1)));
+    for (int w = 0; w < 2; w++) isa[w] = reinterpret_cast<uint32_t *>(take(4 * (n / kIsaStep + 1)));
+    uint2 *text = reinterpret_cast<uint2 *>(take(8 * text_words(n)));
+    uint32_t *lo = reinterpret_cast<uint32_t *>(take(4 * lo_entries(n)));
     cudaError_t e = cudaMemsetAsync(err, 0, 256, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(text, 0, 8 * text_words(n), st);
     if (e != cudaSuccess) return e;
     const uint32_t n_samples = static_cast<uint32_t>(n >> X.sa_shift) + 1u;
-    uint32_t *sa[2];
-    for (int w = 0; w < 2; w++) {
-        sa[w] = reinterpret_cast<uint32_t *>(p);
-        p += derived_align(4 * (n + 1));
+    for (int w = 0; w < 2; w++)
         sa_fill_kernel<<<(n_samples + 255u) / 256u, 256, 0, st>>>(X.t[w], X.sa_shift, 64u << X.sa_shift, n_samples,
-                                                                  sa[w], err);
+                                                                  sa[w], isa[w], w ? nullptr : text + kTextPad, err);
+    const uint32_t depth = lo_depth(n), end = static_cast<uint32_t>(n + 1);
+    if ((e = cudaMemsetAsync(lo, 0, 4, st)) != cudaSuccess) return e;  // no suffix is below the empty string
+    for (uint32_t j = 0; j < depth; j++) {
+        const uint64_t strings = 1ull << (2 * j);
+        lo_level_kernel<<<static_cast<unsigned>((strings + 255) / 256), 256, 0, st>>>(X.t[0], strings, lo);
     }
+    e = cudaMemcpyAsync(lo + lo_entries(n) - 1, &end, 4, cudaMemcpyHostToDevice, st);
     uint32_t bad = 1;
-    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, err, 4, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess || bad) return e;
-    X.sa[0] = sa[0];
-    X.sa[1] = sa[1];
+    for (int w = 0; w < 2; w++) {
+        X.sa[w] = sa[w];
+        X.isa[w] = isa[w];
+    }
+    X.text = text + kTextPad;
+    X.lo = lo;
+    X.lo_k = depth;
     *ok = true;
     return cudaSuccess;
 }

@@ -9,6 +9,14 @@ namespace aln {
 
 struct DIndex;
 
+#ifndef ALN_LO_STRINGS
+#define ALN_LO_STRINGS 4
+#endif
+// Strings in the k-mer table per suffix, at most: with 4 (14-mers at 100 Mbp, 1.1
+// GB) 1 M reads take 3.7 ms, with 1 (13-mers) 4.9 ms, as every part then has a
+// chance place or two.
+constexpr uint64_t kLoStrings = ALN_LO_STRINGS;
+
 constexpr uint64_t derived_align(uint64_t bytes) { return (bytes + 255u) & ~255ull; }
 
 uint64_t derived_bytes(uint64_t n);

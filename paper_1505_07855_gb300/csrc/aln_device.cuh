@@ -22,6 +22,9 @@ namespace aln {
 constexpr uint32_t kRowsPerBlock = 192;
 constexpr uint32_t kHalfRows = 96;
 
+constexpr uint32_t kIsaStep = 4;    // text positions per entry of the derived inverse suffix array
+constexpr uint32_t kTextPad = 16;   // words before and after the text's planes (a read's window may pass its ends)
+
 struct DText {
     const uint4 *blocks;     // 4 x uint4 per 64-byte block: counts, then 12 symbol words
     const uint32_t *sa_samp; // SA[r] for r % sa_sample == 0
@@ -35,7 +38,12 @@ struct DIndex {
     DText t[2];              // t[0] = X, t[1] = X reversed
     uint32_t kmer_k;
     uint32_t sa_shift;       // log2(sa_sample)
-    const uint32_t *sa[2];   // every SA value of X and of X reversed (derived at upload), or nullptr
+    // derived at upload (aln_derive.cu); null and 0 without them
+    const uint32_t *sa[2];   // every SA value of X and of X reversed
+    const uint32_t *isa[2];  // rows of the suffixes at text positions 0, kIsaStep, 2 kIsaStep, ...
+    const uint2 *text;       // X as bit planes (low bits, high bits), 32 bases a word, kTextPad words either side
+    const uint32_t *lo;      // suffixes of X below each string of lo_k bases (first base highest); [4^lo_k] = n + 1
+    uint32_t lo_k;
 };
 
 __device__ __forceinline__ uint4 ld_nc(const uint4 *p) {
@@ -141,17 +149,22 @@ __device__ __forceinline__ void lf1(const DText &T, uint32_t c, uint32_t &lo, ui
 }
 
 // LF(r) = C1[B[r]] + occ_before(B[r], r) for a row r != primary: the row of the
-// suffix that starts one text position earlier.
-__device__ __forceinline__ uint32_t lf_row(const DText &T, uint32_t r) {
+// suffix that starts one text position earlier; c = B[r], the base there.
+__device__ __forceinline__ uint32_t lf_row(const DText &T, uint32_t r, uint32_t &c) {
     const uint32_t b = r / kRowsPerBlock, o = r - b * kRowsPerBlock;
     HalfBlock H;
     load_half(T.blocks, b, o, H);
-    const uint32_t c = sym_in_half(H, o);
+    c = sym_in_half(H, o);
     uint32_t occ[4];
     occ4_in_half(H, o, occ);
     uint32_t v = occ[c];
     if (c == 0) v -= (r > T.primary) ? 1u : 0u;
     return T.C1[c] + v;
+}
+
+__device__ __forceinline__ uint32_t lf_row(const DText &T, uint32_t r) {
+    uint32_t c;
+    return lf_row(T, r, c);
 }
 
 }  // namespace aln

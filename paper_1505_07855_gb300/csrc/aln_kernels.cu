@@ -18,6 +18,7 @@
 
 #include "aln_flat.cuh"
 #include "aln_search.cuh"
+#include "aln_seed.cuh"
 
 namespace aln {
 
@@ -33,17 +34,54 @@ __device__ unsigned long long g_stats[16];
 #define STAT_ADD(i, v) atomicAdd(&g_stats[i], static_cast<unsigned long long>(v))
 #endif
 
+// Whether a search of these limits can be answered from seeds: the derived
+// arrays are there, a transcript has one gap at most, and the caller has set no
+// bound on the tree search's work (its reports are that search's).
+bool seed_supported(const DIndex &X, const SearchParams &p) {
+    return X.lo && min(p.max_gapo, p.z) <= 1u && !p.bounded;
+}
+
+// One thread per read, the tree search; with `seeded`, the block first answers what
+// it can of its reads from seeds, kPlainLanes lanes a read, and its first threads
+// search the rest.  A block then takes a quarter of its threads' number of reads,
+// so that a batch of few reads still has blocks for every SM.
+constexpr int kPlainLanes = 16;
+constexpr uint32_t kPlainReads = kThreads / 4;    // reads of a seeded block
+constexpr uint32_t kPlainTargets = 32, kPlainPlaces = 2048;
+
 template <int STACK_CAP>
 __global__ void __launch_bounds__(kThreads) aln_plain_kernel(DIndex X, ReadBatch rb, uint32_t n_reads, SearchParams p,
-                                                             aln_read_result *res, aln_hit *hits) {
-    __shared__ uint32_t s_bases[kReadWords * kThreads];
-    __shared__ uint32_t s_nmask[kMaskWords * kThreads];
-    const uint32_t r = blockIdx.x * kThreads + threadIdx.x;
-    if (r >= n_reads) return;
+                                                             aln_read_result *res, aln_hit *hits, bool seeded) {
+    __shared__ union {
+        SeedRead<kPlainTargets> read[kThreads / kPlainLanes];
+        struct {
+            uint32_t bases[kReadWords * kThreads], nmask[kMaskWords * kThreads];
+        } tree;
+    } sh;
+    __shared__ uint32_t s_rest[kPlainReads], s_count;
+    uint32_t r;
+    if (seeded) {
+        if (threadIdx.x == 0) s_count = 0;
+        __syncthreads();
+        const uint32_t group = threadIdx.x / kPlainLanes, first = blockIdx.x * kPlainReads;
+        for (uint32_t i = group; i < kPlainReads; i += kThreads / kPlainLanes) {  // the same rounds for every group
+            const bool active = first + i < n_reads;
+            const bool done = seed_search<kPlainLanes, kPlainTargets, false>(X, rb, p, sh.read[group], first + i, active,
+                                                                             kPlainPlaces, res, hits);
+            if (active && !done && threadIdx.x % kPlainLanes == 0) s_rest[atomicAdd(&s_count, 1u)] = first + i;
+        }
+        __syncthreads();
+        if (threadIdx.x >= s_count) return;
+        r = s_rest[threadIdx.x];
+    } else {
+        r = blockIdx.x * kThreads + threadIdx.x;
+        if (r >= n_reads) return;
+    }
     const uint32_t m = rb.len[r];
     const uint32_t z = rb.z ? rb.z[r] : p.z;
-    ReadView rv{s_bases + threadIdx.x, s_nmask + threadIdx.x};
-    if (m <= ALN_MAX_READ_LEN && m > 0) load_read(rb, rb.offset[r], m, s_bases + threadIdx.x, s_nmask + threadIdx.x);
+    ReadView rv{sh.tree.bases + threadIdx.x, sh.tree.nmask + threadIdx.x};
+    if (m <= ALN_MAX_READ_LEN && m > 0)
+        load_read(rb, rb.offset[r], m, sh.tree.bases + threadIdx.x, sh.tree.nmask + threadIdx.x);
     Search<STACK_CAP> S;
     S.run(X, rv, m, z, p, res + r, hits + static_cast<uint64_t>(r) * p.hit_cap);
 }
@@ -57,6 +95,8 @@ __global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_persi
                                                                   SearchParams p, aln_read_result *res,
                                                                   aln_hit *hits, uint32_t *queue,
                                                                   const uint32_t *order, const uint2 *dbp) {
+    // after a seed search that left no read, the queue starts at its end
+    if (__all_sync(0xFFFFFFFFu, *reinterpret_cast<volatile uint32_t *>(queue) >= n_reads)) return;
     __shared__ uint32_t s_bases[kReadWords * kThreads];
     __shared__ uint32_t s_nmask[kMaskWords * kThreads];
     __shared__ uint4 s_stack[SMEM * kThreads];
@@ -251,9 +291,8 @@ __global__ void aln_heavy_start_kernel(SearchParams p, const uint2 *dbp, uint32_
 }
 
 template <int STACK_CAP, bool SCORE>
-__global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_heavy_pass_kernel(DIndex X, ReadBatch rb,
-                                                                                           SearchParams p,
-                                                                                           const uint2 *dbp) {
+__device__ __forceinline__ void heavy_pass(const DIndex &X, const ReadBatch &rb, const SearchParams &p,
+                                           const uint2 *dbp) {
     constexpr int SMEM = kSmemStackDefault;
     __shared__ uint32_t s_bases[kReadWords * kThreads];
     __shared__ uint32_t s_nmask[kMaskWords * kThreads];
@@ -484,6 +523,13 @@ __global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_heavy
         atomicAdd(&H.hdr->lane_trips, static_cast<unsigned long long>(wt));
         atomicAdd(&H.hdr->busy_trips, static_cast<unsigned long long>(wb));
     }
+}
+
+template <int STACK_CAP, bool SCORE>
+__global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_heavy_pass_kernel(DIndex X, ReadBatch rb,
+                                                                                           SearchParams p,
+                                                                                           const uint2 *dbp) {
+    heavy_pass<STACK_CAP, SCORE>(X, rb, p, dbp);
 }
 
 // Score-ordered result of a handed-over read from its tables (the rule of the
@@ -738,23 +784,110 @@ cudaError_t debug_stats(unsigned long long *out, int reset) {
 // t >> 1 on that strand's other index (strand 0 on X, strand 1 on X reversed)
 // and stores its breakpoints; reads the search would flag before any scan get
 // zeros.  The persistent search then starts from these instead of scanning.
+__device__ __forceinline__ void dscan_one(const DIndex &X, const ReadBatch &rb, const SearchParams &p, uint32_t r,
+                                          uint32_t s, uint32_t *sb, uint32_t *sn, uint2 *dbp) {
+    const uint32_t m = rb.len[r];
+    const uint32_t z = rb.z ? rb.z[r] : p.z;
+    uint2 out = make_uint2(0u, 0u);
+    if (m >= 1 && m <= ALN_MAX_READ_LEN && z <= ALN_MAX_Z && z <= p.z) {
+        load_read(rb, rb.offset[r], m, sb, sn);
+        const ReadView rv{sb, sn};
+        d_scan(X.t[s], rv, m, s, min(z + 1, 8u), out.x, out.y);
+    }
+    dbp[2ull * r + s] = out;
+}
+
 __global__ void __launch_bounds__(kThreads) aln_dscan_kernel(DIndex X, ReadBatch rb, uint32_t n, SearchParams p,
                                                              uint2 *dbp) {
     __shared__ uint32_t s_bases[kReadWords * kThreads];
     __shared__ uint32_t s_nmask[kMaskWords * kThreads];
     const uint64_t t = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x;
     if (t >= 2ull * n) return;
-    const uint32_t r = static_cast<uint32_t>(t >> 1), s = static_cast<uint32_t>(t & 1u);
-    const uint32_t m = rb.len[r];
-    const uint32_t z = rb.z ? rb.z[r] : p.z;
-    uint2 out = make_uint2(0u, 0u);
-    if (m >= 1 && m <= ALN_MAX_READ_LEN && z <= ALN_MAX_Z && z <= p.z) {
-        uint32_t *sb = s_bases + threadIdx.x, *sn = s_nmask + threadIdx.x;
-        load_read(rb, rb.offset[r], m, sb, sn);
-        const ReadView rv{sb, sn};
-        d_scan(X.t[s], rv, m, s, min(z + 1, 8u), out.x, out.y);
+    dscan_one(X, rb, p, static_cast<uint32_t>(t >> 1), static_cast<uint32_t>(t & 1u), s_bases + threadIdx.x,
+              s_nmask + threadIdx.x, dbp);
+}
+
+// ---------------------------------------------------------------- seed search
+//
+// aln_seed_kernel answers the reads whose parts lead to few places (see
+// aln_seed.cuh), G lanes a read; aln_seed_wide_kernel takes the reads it leaves,
+// a warp each with room for kCandCap targets; aln_dscan_list_kernel scans the D
+// arrays of what is left then, which the persistent search and the heavy phase
+// search as before: the rest fills the visit order from its end, and the queue
+// starts where it begins.  The lists and their counts stay on the device.
+
+struct SeedCounts {          // in the scratch's first words, cleared before the call's kernels
+    uint32_t wide, taken;    // reads left by the first kernel; those the second has taken up
+    uint32_t rest;           // reads left for the tree search
+};
+
+// Room for targets and places to look at, first for a read's 8 or 16 lanes: past
+// that the other reads of the warp wait for it, so it goes to a warp of its own.
+// There, kCandCap targets are what the tree search keeps, and 16384 places are half
+// a millisecond of a warp, about what the tree search of such a read costs.
+constexpr uint32_t kSeedTargets = 32;
+constexpr uint32_t kSeedPlaces = 256;
+constexpr uint32_t kWidePlaces = 16384;
+
+// Resident blocks per SM: 4 / 5 / 6 take 4.2 / 3.97 / 3.89 ms for 1 M reads of 100
+// bases on 100 Mbp (latency; 6 spills 30 bytes in the gapped path), the wide kernel
+// gains nothing past 5.
+#ifndef ALN_SEED_MIN_BLOCKS
+#define ALN_SEED_MIN_BLOCKS 6
+#endif
+#ifndef ALN_WIDE_MIN_BLOCKS
+#define ALN_WIDE_MIN_BLOCKS 5
+#endif
+
+template <int G, bool SCORE>
+__global__ void __launch_bounds__(kThreads, ALN_SEED_MIN_BLOCKS) aln_seed_kernel(DIndex X, ReadBatch rb, uint32_t n, SearchParams p,
+                                                            aln_read_result *res, aln_hit *hits, SeedCounts *counts,
+                                                            uint32_t *wide) {
+    __shared__ SeedRead<kSeedTargets> s_read[kThreads / G];
+    if (blockIdx.x == 0 && p.heavy.hdr && threadIdx.x < sizeof(HeavyHdr) / 4)  // what the heavy phase counts in
+        reinterpret_cast<uint32_t *>(p.heavy.hdr)[threadIdx.x] = 0;
+    const uint64_t r = (static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x) / G;
+    const bool active = r < n;
+    const bool done = seed_search<G, kSeedTargets, SCORE>(X, rb, p, s_read[threadIdx.x / G], static_cast<uint32_t>(r),
+                                                          active, kSeedPlaces, res, hits);
+    if (active && !done && (threadIdx.x & (G - 1)) == 0) wide[atomicAdd(&counts->wide, 1u)] = static_cast<uint32_t>(r);
+}
+
+template <bool SCORE>
+__global__ void __launch_bounds__(kThreads, ALN_WIDE_MIN_BLOCKS) aln_seed_wide_kernel(DIndex X, ReadBatch rb, SearchParams p,
+                                                                 aln_read_result *res, aln_hit *hits,
+                                                                 SeedCounts *counts, const uint32_t *wide,
+                                                                 uint32_t *order_end) {
+    __shared__ SeedRead<kCandCap> s_read[kThreads / 32];
+    const uint32_t lane = threadIdx.x & 31u, n = counts->wide;
+    for (;;) {
+        uint32_t i = 0;
+        if (lane == 0) i = atomicAdd(&counts->taken, 1u);
+        i = __shfl_sync(0xFFFFFFFFu, i, 0);
+        if (i >= n) break;
+        const uint32_t r = wide[i];
+        const bool done = seed_search<32, kCandCap, SCORE>(X, rb, p, s_read[threadIdx.x / 32], r, true, kWidePlaces, res,
+                                                           hits);
+        if (!done && lane == 0) *(order_end - 1 - atomicAdd(&counts->rest, 1u)) = r;
     }
-    dbp[t] = out;
+}
+
+__global__ void __launch_bounds__(kThreads) aln_dscan_list_kernel(DIndex X, ReadBatch rb, SearchParams p,
+                                                                  uint32_t n_reads, const uint32_t *order,
+                                                                  const SeedCounts *counts, uint32_t *queue,
+                                                                  uint2 *dbp) {
+    __shared__ uint32_t s_bases[kReadWords * kThreads];
+    __shared__ uint32_t s_nmask[kMaskWords * kThreads];
+    const uint32_t n = counts->rest;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *queue = n_reads - n;
+    if (n == 0) return;
+    const uint64_t step = static_cast<uint64_t>(gridDim.x) * kThreads;
+    const uint64_t first = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x;
+    if (p.heavy.hdr)  // the heavy phase's ready words, cleared only when it may run
+        for (uint64_t t = first; t < kHeavyPool; t += step) p.heavy.ready[t] = 0;
+    for (uint64_t t = first; t < 2ull * n; t += step)
+        dscan_one(X, rb, p, order[n_reads - n + (t >> 1)], static_cast<uint32_t>(t & 1u), s_bases + threadIdx.x, s_nmask + threadIdx.x,
+                  dbp);
 }
 
 // Visit order for the persistent search: reads by decreasing lower bound
@@ -811,8 +944,9 @@ static cudaError_t launch_cap(const DIndex &X, const ReadBatch &rb, uint32_t n, 
                               aln_read_result *res, aln_hit *hits, uint32_t mode, uint32_t *queue,
                               void *scratch, cudaStream_t st) {
     if (mode == ALN_MODE_PLAIN) {
-        const uint32_t blocks = (n + kThreads - 1) / kThreads;
-        aln_plain_kernel<CAP><<<blocks, kThreads, 0, st>>>(X, rb, n, p, res, hits);
+        const bool seeded = seed_supported(X, p);
+        const uint32_t each = seeded ? kPlainReads : kThreads;
+        aln_plain_kernel<CAP><<<(n + each - 1) / each, kThreads, 0, st>>>(X, rb, n, p, res, hits, seeded);
     } else {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
@@ -823,12 +957,34 @@ static cudaError_t launch_cap(const DIndex &X, const ReadBatch &rb, uint32_t n, 
         uint32_t blocks = static_cast<uint32_t>(sms * per_sm);
         const uint32_t need = (n + kThreads - 1) / kThreads;
         if (blocks > need) blocks = need ? need : 1;
-        cudaMemsetAsync(queue, 0, sizeof(uint32_t), st);
         uint2 *dbp = nullptr;
         uint32_t *order = nullptr;
         SearchParams pp = p;
         pp.heavy.hdr = nullptr;
-        if (scratch) {  // D pre-pass and visit order (layout: search_scratch_bytes)
+        const bool seeded = scratch && seed_supported(X, p);
+        if (seeded) {
+            // the first list takes the D breakpoints' place, which are written after it is read
+            SeedCounts *counts = static_cast<SeedCounts *>(scratch);
+            dbp = reinterpret_cast<uint2 *>(static_cast<char *>(scratch) + 256);
+            order = reinterpret_cast<uint32_t *>(static_cast<char *>(scratch) + 256 + 16ull * n);
+            uint32_t *wide = reinterpret_cast<uint32_t *>(dbp);
+            if (p.heavy_after != 0xFFFFFFFFu) pp.heavy = heavy_layout(scratch, n);
+            cudaMemsetAsync(counts, 0, sizeof(SeedCounts), st);
+            // parts of both strands on 8 lanes for z <= 3, else on 16
+            if (p.z <= 3)
+                aln_seed_kernel<8, SCORE><<<static_cast<unsigned>((8ull * n + kThreads - 1) / kThreads), kThreads, 0, st>>>(
+                    X, rb, n, pp, res, hits, counts, wide);
+            else
+                aln_seed_kernel<16, SCORE><<<static_cast<unsigned>((16ull * n + kThreads - 1) / kThreads), kThreads, 0, st>>>(
+                    X, rb, n, pp, res, hits, counts, wide);
+            const uint32_t wb = min((n + 3u) / 4u, static_cast<uint32_t>(sms) * 6u);
+            aln_seed_wide_kernel<SCORE><<<wb, kThreads, 0, st>>>(X, rb, pp, res, hits, counts, wide, order + n);
+            const uint32_t db = min(static_cast<uint32_t>((2ull * n + kThreads - 1) / kThreads), static_cast<uint32_t>(sms) * 8u);
+            aln_dscan_list_kernel<<<db, kThreads, 0, st>>>(X, rb, pp, n, order, counts, queue, dbp);
+        } else {
+            cudaMemsetAsync(queue, 0, sizeof(uint32_t), st);
+        }
+        if (scratch && !seeded) {  // D pre-pass and visit order (layout: search_scratch_bytes)
             uint32_t *counts = static_cast<uint32_t *>(scratch), *cursor = counts + kOrderBins;
             dbp = reinterpret_cast<uint2 *>(static_cast<char *>(scratch) + 256);
             order = reinterpret_cast<uint32_t *>(static_cast<char *>(scratch) + 256 + 16ull * n);

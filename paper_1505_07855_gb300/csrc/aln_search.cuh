@@ -98,6 +98,7 @@ struct SearchParams {
     uint32_t help_after;            // persistent form: expansions after which a read takes idle lanes
     uint32_t heavy_after;           // persistent form: owner expansions after which a read goes to the heavy phase
     uint32_t sc_mm, sc_go, sc_ge, max_best;  // score-ordered mode: penalties and the cap on best places
+    uint32_t bounded;               // the caller set a work or loop limit
     HeavyCtx heavy;                 // heavy phase state (hdr == nullptr: no heavy phase)
     unsigned long long loop_limit;  // persistent form: loop trips per warp
     uint32_t *status;               // ALN_STATUS_* bits, or nullptr

@@ -1,0 +1,793 @@
+// Seed-and-verify search (sm_103a): the reads whose error-free parts lead to few
+// places in the text are answered from those places; the tree search is left the
+// rest.
+//
+// A transcript with at most b differences, cut at b + 1 parts of the read, leaves
+// one part without any: that part occurs in the text as it is, on the
+// transcript's diagonal.  So every place of every part, looked at base by base,
+// gives every target within b differences.  With at most one gap a transcript is
+// a prefix on one diagonal, a run of inserted or deleted bases, and a suffix on
+// another; its target is (start on the first, end on the second), and the fewest
+// mismatches over the gap's places is the target's least witness, as the other
+// terms of the witness follow from the gap's length.  The search's limits (gap
+// and seed limits, end window, N) are those of aln_search.cuh, read index p of
+// the reverse strand being pattern index m - 1 - p here.  Both strands work on X:
+// the reverse strand's pattern is the reverse complement of the read.
+//
+// A target's rows in the suffix array of its strand's text come from the derived
+// inverse (its sampled entries and at most three LF steps).  All places of a
+// target are found, so equal targets, which are neighbours in the suffix array,
+// give its interval; targets of different lengths with the same interval merge as
+// in the tree search.
+//
+// G lanes a read: one lane per (strand, part) finds the part's rows (one look-up
+// in the table of k-mers, a few LF steps in a repeat), then the lanes share the
+// places out.
+//
+// Where the tree search of a read of 100 bases expands about 1900 nodes, one after
+// the other, this takes 2 (z + 1) look-ups at once and looks at about ten places
+// (100 Mbp), each a read of the suffix array and of the text.  1 M reads of 100
+// bases at z = 4 on 100 Mbp: 64.9 -> 3.9 ms; 400 000 reads of 36 to 250 bases on
+// 3.1 Gbp: 736 -> 20 ms (profiles/aln_seed.md).  It is bound by the latency of
+// those four dependent random reads and by instruction issue, not by bandwidth.
+#pragma once
+
+#include <cstdint>
+
+#include "aln_search.cuh"
+
+namespace aln {
+
+#ifndef ALN_EXTEND
+#define ALN_EXTEND 24
+#endif
+// Bases a part grows by at most, past the table's: 300 000 mates on 3.1 Gbp take
+// 8.03 / 7.54 / 7.28 ms with 6 / 12 / 24, unique reads do not grow at all.
+constexpr int kExtend = ALN_EXTEND;
+constexpr uint32_t kWideRows = 1u << 20;  // a part's rows saturate here
+#ifndef ALN_MANY_PLACES
+#define ALN_MANY_PLACES 3
+#endif
+// Places per lane from which a pass starts over with fewer, longer parts.  1, 2, 3, 6
+// and 8 are within 2 % of each other on the 3.1 Gbp batches (1 costs unique reads
+// of 100 Mbp 12 %).
+constexpr uint32_t kManyPlaces = ALN_MANY_PLACES;
+
+// Symbols c in B[0 .. pos-1] of one base.
+__device__ __forceinline__ uint32_t occ1(const DText &T, uint32_t c, uint32_t pos) {
+    const uint32_t b = pos / kRowsPerBlock, o = pos - b * kRowsPerBlock;
+    HalfBlock H;
+    load_half(T.blocks, b, o, H);
+    const bool up = o >= kHalfRows;
+    const int x = static_cast<int>(up ? o - kHalfRows : o);
+    const uint32_t fl = (c & 1u) ? 0u : 0xFFFFFFFFu, fh = (c & 2u) ? 0u : 0xFFFFFFFFu;
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int g = 0; g < 3; g++) {
+        uint32_t m = __funnelshift_lc(0xFFFFFFFFu, 0u, static_cast<uint32_t>(max(x - 32 * g, 0)));
+        if (!up) m = ~m;
+        cnt += __popc((H.w[g] ^ fl) & (H.w[3 + g] ^ fh) & m);
+    }
+    const uint32_t base = c == 0 ? H.cnt[0] : (c == 1 ? H.cnt[1] : (c == 2 ? H.cnt[2] : H.cnt[3]));
+    const uint32_t v = up ? base + cnt : base - cnt;
+    return c == 0 && pos > T.primary ? v - 1u : v;
+}
+
+// Row of the suffix of text w that starts at position pos (0 .. n).
+__device__ __forceinline__ uint32_t row_of(const DIndex &X, int w, uint32_t pos) {
+    const DText &T = X.t[w];
+    const uint64_t s = (static_cast<uint64_t>(pos) + kIsaStep - 1) / kIsaStep;
+    const uint64_t at = s * kIsaStep;
+    uint32_t row = 0, steps = T.n - pos;  // past the last sampled position: from the suffix "$", row 0
+    if (at <= T.n) {
+        row = __ldg(X.isa[w] + s);
+        steps = static_cast<uint32_t>(at) - pos;
+    }
+    for (; steps; steps--) row = lf_row(T, row);
+    return row;
+}
+
+__device__ __forceinline__ uint32_t low_mask(int k) {  // the low k bits, k clamped to 0..32
+    return __funnelshift_lc(0xFFFFFFFFu, 0u, static_cast<uint32_t>(max(k, 0)));
+}
+
+// Bits [from, to) of a read's mask that fall into its word w.
+__device__ __forceinline__ uint32_t span_mask(int from, int to, int w) {
+    return low_mask(to - 32 * w) & ~low_mask(from - 32 * w);
+}
+
+constexpr int kPlaneWords = 8;  // words of a mask of ALN_MAX_READ_LEN bases
+
+// A pattern (a read on one strand, in text order) as bit planes in shared memory.
+struct Pattern {
+    uint32_t lo[kPlaneWords], hi[kPlaneWords], nn[kPlaneWords];
+};
+
+// mis = the pattern's mismatches (bit j = pattern index j) with the pattern's
+// first base on text position x.
+__device__ __forceinline__ void mismatches(const uint2 *text, const Pattern &P, long long x, int m,
+                                           uint32_t mis[kPlaneWords]) {
+    const uint2 *t = text + (x >> 5);
+    const uint32_t s = static_cast<uint32_t>(x & 31);
+    uint2 a = __ldg(t);
+#pragma unroll
+    for (int w = 0; w < kPlaneWords; w++) {
+        mis[w] = 0;
+        if (32 * w < m) {
+            const uint2 b = __ldg(t + w + 1);
+            const uint32_t lo = __funnelshift_r(a.x, b.x, s), hi = __funnelshift_r(a.y, b.y, s);
+            mis[w] = ((lo ^ P.lo[w]) | (hi ^ P.hi[w]) | P.nn[w]) & low_mask(m - 32 * w);
+            a = b;
+        }
+    }
+}
+
+__device__ __forceinline__ uint32_t count_in(const uint32_t mis[kPlaneWords], int from, int to) {
+    uint32_t c = 0;
+#pragma unroll
+    for (int w = 0; w < kPlaneWords; w++) {
+        if (32 * w >= to) break;
+        c += __popc(mis[w] & span_mask(from, to, w));
+    }
+    return c;
+}
+
+// Index of the (r + 1)-th mismatch from the start (m if there are fewer).
+__device__ __forceinline__ int nth_low(const uint32_t mis[kPlaneWords], uint32_t r, int m) {
+    uint32_t x = 0;
+    int at = -1;
+#pragma unroll
+    for (int w = 0; w < kPlaneWords; w++) {
+        if (32 * w >= m) break;
+        const uint32_t c = __popc(mis[w]);
+        if (at < 0) {
+            if (r < c) {
+                x = mis[w];
+                at = 32 * w;
+            } else {
+                r -= c;
+            }
+        }
+    }
+    if (at < 0) return m;
+    for (; r; r--) x &= x - 1;
+    return at + __ffs(x) - 1;
+}
+
+// Index of the (r + 1)-th mismatch from the end (-1 if there are fewer).
+__device__ __forceinline__ int nth_high(const uint32_t mis[kPlaneWords], uint32_t r) {
+    uint32_t x = 0;
+    int at = -1;
+#pragma unroll
+    for (int w = kPlaneWords - 1; w >= 0; w--) {
+        const uint32_t c = __popc(mis[w]);
+        if (at < 0) {
+            if (r < c) {
+                x = mis[w];
+                at = 32 * w;
+            } else {
+                r -= c;
+            }
+        }
+    }
+    if (at < 0) return -1;
+    for (; r; r--) x &= ~(0x80000000u >> __clz(x));
+    return at + 31 - __clz(x);
+}
+
+// The places of one gap of length g between a prefix with mismatches A and a
+// suffix with mismatches B (a deletion, or an insertion of pattern bases
+// [p, p + g)): the fewest mismatches over p in [plo, phi] that keep the seed
+// limit, or none (> most).  Only the few gap lengths whose diagonals both match
+// come past the two bounds below, so the walk over p is rare and short.
+struct SeedZone {
+    int from, to;      // pattern indices of the seed ([0, 0): no seed)
+    uint32_t most;     // differences allowed in it
+    bool reverse;      // the pattern is the reverse complement
+};
+
+__device__ __forceinline__ uint32_t best_gap(const uint32_t A[kPlaneWords], const uint32_t B[kPlaneWords], int m, int g,
+                                             bool del, int plo, int phi, uint32_t most, const SeedZone &Z) {
+    constexpr uint32_t kNone = 0xFFFFFFFFu;
+    const int gi = del ? 0 : g;
+    phi = min(phi, nth_low(A, most, m));           // the prefix has at most `most` mismatches
+    plo = max(plo, nth_high(B, most) + 1 - gi);    // and so has the suffix
+    if (plo > phi) return kNone;
+    uint32_t a[kPlaneWords], b[kPlaneWords];
+#pragma unroll
+    for (int w = 0; w < kPlaneWords; w++) {
+        a[w] = A[w];
+        b[w] = B[w];
+    }
+    uint32_t f = count_in(A, 0, plo) + count_in(B, plo + gi, m);
+    uint32_t sa = 0, sb = 0;
+    const bool seeded = Z.to > Z.from;
+    if (seeded) {
+        sa = count_in(A, Z.from, min(Z.to, plo));
+        sb = count_in(B, max(Z.from, plo + gi), Z.to);
+    }
+    uint32_t best = kNone;
+    for (int p = plo;; p++) {
+        bool ok = f <= most && f < best;
+        if (ok && seeded) {
+            // gap bases in the seed: inserted bases by index; a deletion at the
+            // read index that follows it (p on the forward strand, and p - 1 in
+            // pattern order on the reverse strand)
+            const int at = Z.reverse ? p - 1 : p;
+            const int in = del ? (at >= Z.from && at < Z.to ? g : 0) : max(0, min(Z.to, p + g) - max(Z.from, p));
+            ok = sa + sb + static_cast<uint32_t>(in) <= Z.most;
+        }
+        if (ok) best = f;
+        if (p >= phi) break;
+        const uint32_t ia = (a[p >> 5] >> (p & 31)) & 1u, q = static_cast<uint32_t>(p + gi);
+        const uint32_t ib = (b[q >> 5] >> (q & 31u)) & 1u;  // q < m: p < phi <= m - gi
+        f += ia - ib;
+        if (seeded) {
+            if (p >= Z.from && p < Z.to) sa += ia;
+            if (static_cast<int>(q) >= Z.from && static_cast<int>(q) < Z.to) sb -= ib;
+        }
+    }
+    return best;
+}
+
+// Whether diagonal d can be the prefix (or, `ahead`, the suffix) of a target with
+// a gap: its own mismatches and the end window bound the gap's place, and the
+// bases past that place (of them, the 32 at the read's far end) have to fit a
+// neighbouring diagonal.  One word a diagonal in the lane that found d, against
+// the masks of the whole read by all lanes: what has no indel ends here, both the
+// copies of a repeat and the read's own place.
+__device__ __forceinline__ bool gap_fits(const uint2 *text, const Pattern &P, long long d, int m,
+                                         const uint32_t mis[kPlaneWords], int F, int gmost, int e, bool ahead) {
+    const int i = ahead ? 0 : max(m - 32, 0), w = i >> 5;
+    const uint32_t s = static_cast<uint32_t>(i & 31);
+    const int v = min(w + 1, kPlaneWords - 1);
+    const uint32_t lo = __funnelshift_r(P.lo[w], P.lo[v], s), hi = __funnelshift_r(P.hi[w], P.hi[v], s);
+    const uint32_t nn = __funnelshift_r(P.nn[w], P.nn[v], s);
+    const int bound = ahead ? nth_high(mis, F - 1) + 1 : nth_low(mis, F - 1, m);
+    for (int q = 0; q < 2 * gmost; q++) {
+        const int g = (q >> 1) + 1;
+        const bool del = q & 1;
+        const int window = del ? max(e, 1) : e, gi = del ? 0 : g;
+        const uint32_t zone = ahead ? low_mask(max(bound - gi, window))
+                                    : low_mask(m - i) & ~low_mask(min(bound, m - window - gi) + gi - i);
+        const long long x = d + i + (del != ahead ? g : -g);
+        const uint2 a = __ldg(text + (x >> 5)), b = __ldg(text + (x >> 5) + 1);
+        const uint32_t t = static_cast<uint32_t>(x & 31);
+        const uint32_t far = (__funnelshift_r(a.x, b.x, t) ^ lo) | (__funnelshift_r(a.y, b.y, t) ^ hi) | nn;
+        if (__popc(far & zone) + g <= F) return true;
+    }
+    return false;
+}
+
+// Shared memory of one read's lanes.
+template <int E>
+struct SeedRead {
+    Pattern pat[2];
+    uint32_t bases[18];              // the read, 2 bits a base (two words past it)
+    uint32_t count;                  // targets found (may pass E)
+    uint32_t start[E], key[E];       // target start in X; the tree search's candidate key
+    uint32_t row[E], end[E];         // its rows [row, end); end 0: dropped, or another target stands for them
+};
+
+// `width` low-order bases from index i of the packed read.
+__device__ __forceinline__ uint32_t bases_at(const uint32_t *bases, uint32_t i, uint32_t width) {
+    const uint32_t w = i >> 4, s = 2 * (i & 15u);
+    const uint32_t v = __funnelshift_r(bases[w], bases[w + 1], s);
+    return v & low_mask(static_cast<int>(2 * width));
+}
+
+// Base order reversed in the low `width` bases.
+__device__ __forceinline__ uint32_t reverse_bases(uint32_t v, uint32_t width) {
+    const uint32_t r = __brev(v);
+    const uint32_t x = ((r & 0x55555555u) << 1) | ((r >> 1) & 0x55555555u);
+    return width ? x >> (32u - 2u * width) : 0u;
+}
+
+// Even and odd bits of a word, each as 16 bits.
+__device__ __forceinline__ uint32_t even_bits(uint32_t x) {
+    x &= 0x55555555u;
+    x = (x | (x >> 1)) & 0x33333333u;
+    x = (x | (x >> 2)) & 0x0F0F0F0Fu;
+    x = (x | (x >> 4)) & 0x00FF00FFu;
+    return (x | (x >> 8)) & 0x0000FFFFu;
+}
+
+template <int G>
+__device__ __forceinline__ uint32_t group_min(uint32_t v) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) v = min(v, __shfl_xor_sync(0xFFFFFFFFu, v, o, G));
+    return v;
+}
+
+template <int G>
+__device__ __forceinline__ uint32_t group_sum(uint32_t v) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o, G);
+    return v;
+}
+
+// X[a .. a+L) == X[b .. b+L)
+__device__ __forceinline__ bool same_text(const uint2 *text, uint32_t a, uint32_t b, uint32_t L) {
+    const uint2 *ta = text + (a >> 5), *tb = text + (b >> 5);
+    const uint32_t sa = a & 31u, sb = b & 31u;
+    for (uint32_t w = 0; 32 * w < L; w++) {
+        const uint2 a0 = __ldg(ta + w), a1 = __ldg(ta + w + 1), b0 = __ldg(tb + w), b1 = __ldg(tb + w + 1);
+        const uint32_t d = (__funnelshift_r(a0.x, a1.x, sa) ^ __funnelshift_r(b0.x, b1.x, sb)) |
+                           (__funnelshift_r(a0.y, a1.y, sa) ^ __funnelshift_r(b0.y, b1.y, sb));
+        if (d & low_mask(static_cast<int>(L - 32 * w))) return false;
+    }
+    return true;
+}
+
+__device__ __forceinline__ uint32_t key_diffs(uint32_t key) { return (key >> 28) & 7u; }
+
+__device__ __forceinline__ uint32_t key_score(const SearchParams &p, uint32_t key) {
+    return p.sc_mm * ((key >> 16) & 15u) + p.sc_go * ((key >> 24) & 15u) + p.sc_ge * ((key >> 20) & 15u);
+}
+
+// A target found: recorded unless it is among the first `have`, those of the
+// rounds before (two lanes may record it in one round; the reduction drops the
+// second).
+template <int E>
+__device__ __forceinline__ void add_target(SeedRead<E> &S, uint32_t have, uint32_t strand, long long a, uint32_t len,
+                                           uint32_t mm, uint32_t g) {
+    const uint32_t key = (strand << 31) | ((mm + g) << 28) | ((g ? 1u : 0u) << 24) | ((g ? g - 1u : 0u) << 20) |
+                         (mm << 16) | len;
+    const uint32_t at = static_cast<uint32_t>(a);
+    for (uint32_t j = 0; j < have; j++)
+        if (S.start[j] == at && S.key[j] == key) return;
+    const uint32_t j = atomicAdd(&S.count, 1u);
+    if (j < E) {
+        S.start[j] = at;
+        S.key[j] = key;
+    }
+}
+
+__device__ __forceinline__ void put_hit(aln_hit *to, uint32_t k, uint32_t l, uint32_t key) {
+    aln_hit h;
+    h.k = k;
+    h.l = l;
+    h.aligned_len = static_cast<uint16_t>(key & 0xFFFFu);
+    h.strand = static_cast<uint8_t>(key >> 31);
+    h.n_diff = static_cast<uint8_t>(key_diffs(key));
+    h.n_mm = static_cast<uint8_t>((key >> 16) & 15u);
+    h.n_gapo = static_cast<uint8_t>((key >> 24) & 15u);
+    h.n_gape = static_cast<uint8_t>((key >> 20) & 15u);
+    h.reserved = 0;
+    *to = h;
+}
+
+template <bool SCORE>
+__device__ __forceinline__ void empty_result(aln_read_result *to, uint32_t flags) {
+    aln_read_result out;
+    out.c0 = out.c1 = 0;
+    out.n_hits = 0;
+    out.flags = static_cast<uint8_t>(flags);
+    out.d_best = 255;
+    out.best_score = SCORE ? 255 : 0;
+    *to = out;
+}
+
+// Search of one read by the G lanes of a group; all 32 lanes of the warp call it
+// together (other groups with their own reads, or with active = false).  True
+// if the read's result was written; false if it has too many places or targets
+// for this form (nothing is written then).
+template <int G, int E, bool SCORE>
+__device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchParams &p, SeedRead<E> &S, uint32_t r,
+                            bool active, uint32_t max_places, aln_read_result *res, aln_hit *hits) {
+    constexpr unsigned FULL = 0xFFFFFFFFu;
+    constexpr uint32_t kHalf = G / 2;
+    const uint32_t l = threadIdx.x & (G - 1);
+    const uint32_t n = X.t[0].n;
+    int m = 0;
+    uint32_t z = 0;
+    bool answer = false;  // a read that is not searched: its (empty) result is known
+    uint32_t flags = 0;
+    if (active) {
+        m = rb.len[r];
+        z = rb.z ? rb.z[r] : p.z;
+        if (m > ALN_MAX_READ_LEN) flags |= ALN_FLAG_READ_TOO_LONG;
+        if (z > ALN_MAX_Z || z > p.z) flags |= ALN_FLAG_BAD_LIMIT;
+        answer = flags || m == 0;
+        if (answer) m = 0;
+    }
+    const bool search = active && !answer;
+    // ---- the read into shared memory: packed, and as planes of both strands
+    __syncwarp();
+    if (search) {
+        const uint64_t off = rb.offset[r], last = (off + m - 1) >> 4;
+        for (uint32_t w = l; w < 18; w += G) {
+            uint32_t v = 0;
+            if (16 * w < static_cast<uint32_t>(m)) {
+                const uint64_t at = (off >> 4) + w;
+                const uint32_t a = __ldg(rb.bases + at), b = at + 1 <= last ? __ldg(rb.bases + at + 1) : 0u;
+                v = __funnelshift_r(a, b, 2 * static_cast<uint32_t>(off & 15u));
+            }
+            S.bases[w] = v;
+        }
+        const uint64_t nlast = (off + m - 1) >> 5;
+        for (uint32_t w = l; w < kPlaneWords; w += G) {
+            uint32_t v = 0;
+            if (rb.nmask && 32 * w < static_cast<uint32_t>(m)) {
+                const uint64_t at = (off >> 5) + w;
+                const uint32_t a = __ldg(rb.nmask + at), b = at + 1 <= nlast ? __ldg(rb.nmask + at + 1) : 0u;
+                v = __funnelshift_r(a, b, static_cast<uint32_t>(off & 31u));
+            }
+            S.pat[0].nn[w] = v & low_mask(m - static_cast<int>(32 * w));
+        }
+        if (l == 0) S.count = 0;
+    }
+    __syncwarp();
+    if (search)
+        for (uint32_t w = l; w < kPlaneWords; w += G) {
+            const uint32_t a = S.bases[2 * w], b = S.bases[2 * w + 1];
+            S.pat[0].lo[w] = even_bits(a) | (even_bits(b) << 16);
+            S.pat[0].hi[w] = even_bits(a >> 1) | (even_bits(b >> 1) << 16);
+        }
+    __syncwarp();
+    if (search)
+        for (uint32_t w = l; w < kPlaneWords; w += G) {
+            // pattern index 32 w + i of the reverse strand is read index m - 1 - 32 w - i:
+            // read bits [m - 32 - 32 w, m - 32 w), in reverse
+            const int at = m - 32 - 32 * static_cast<int>(w);
+            const int q = at >> 5;
+            const uint32_t s = static_cast<uint32_t>(at & 31);
+            uint32_t v[3];
+#pragma unroll
+            for (int t = 0; t < 3; t++) {
+                const uint32_t *src = t == 0 ? S.pat[0].lo : (t == 1 ? S.pat[0].hi : S.pat[0].nn);
+                const uint32_t x0 = q >= 0 && q < kPlaneWords ? src[q] : 0u;
+                const uint32_t x1 = q + 1 >= 0 && q + 1 < kPlaneWords ? src[q + 1] : 0u;
+                v[t] = __brev(__funnelshift_r(x0, x1, s));
+            }
+            S.pat[1].lo[w] = ~v[0];
+            S.pat[1].hi[w] = ~v[1];
+            S.pat[1].nn[w] = v[2];
+        }
+    __syncwarp();
+
+    const uint32_t strand = l / kHalf, part = l % kHalf;
+    const uint32_t K = X.lo_k;
+    const bool exhaustive = p.strata != ALN_STRATA_BEST1;
+    const unsigned group_lanes = (G == 32 ? FULL : ((1u << (G & 31)) - 1u)) << ((threadIdx.x & 31u) / G * G);
+    auto zone = [&](uint32_t s) {
+        const int len = min(m, static_cast<int>(p.seed_len));
+        return SeedZone{s ? m - len : 0, s ? m : len, p.seed_z, s != 0};
+    };
+    // ---- passes: every target within b differences.  b = z at once where the parts
+    // are long enough to be rare; else, or where they still turn out to have many
+    // places (a repeat), few long parts first: what they find bounds the
+    // differences that the next pass has to look for.
+    uint32_t b = z;
+    bool stepping = exhaustive;  // b starts from 1 and grows by one (or, of an exhaustive search, is z)
+    if (!exhaustive && static_cast<uint32_t>(m) < (z + 1) * K) {
+        const uint32_t fit = static_cast<uint32_t>(m) / K;
+        b = min(z, fit > 2 ? fit - 1 : 1u);
+    }
+    uint32_t F = z;            // differences a target may still have
+    uint32_t dmin = 255;       // fewest found
+    bool todo = search, failed = false;
+    while (__any_sync(FULL, todo)) {
+        // the rows of this lane's part
+        uint32_t lo = 0, hi = 0, width = 0, ps = 0, pe = 0, off = 0;  // part [ps, pe) and first matched base, in pattern order
+        uint32_t next = 0, bases = 0;                                 // read index of the next base outside, bases left
+        if (todo && part <= b) {
+            const uint32_t s0 = static_cast<uint32_t>(m) * part / (b + 1);
+            const uint32_t s1 = static_cast<uint32_t>(m) * (part + 1) / (b + 1);
+            ps = strand ? m - s1 : s0;
+            pe = strand ? m - s0 : s1;
+            bool clean = true;
+            for (uint32_t w = s0 >> 5; 32 * w < s1; w++)
+                clean = clean && !(S.pat[0].nn[w] & span_mask(static_cast<int>(s0), static_cast<int>(s1), static_cast<int>(w)));
+            if (s1 == s0) {
+                width = kWideRows;
+            } else if (clean) {
+                const uint32_t kk = min(K, s1 - s0);
+                uint64_t id;  // the part's last kk bases in text order, first base highest
+                if (strand) id = ~bases_at(S.bases, s0, kk) & low_mask(static_cast<int>(2 * kk));
+                else id = reverse_bases(bases_at(S.bases, s1 - kk, kk), kk);
+                const uint32_t sh = 2 * (K - kk);
+                hi = __ldg(X.lo + ((id + 1) << sh));
+                lo = __ldg(X.lo + (id << sh));
+                // a shorter string's rows also hold the suffixes that end within K
+                // bases, which sort below its first K-mer: at most one per length
+                lo -= min(lo, K - kk);
+                off = pe - kk;
+                width = hi > lo ? min(hi - lo, kWideRows) : 0u;
+                bases = s1 - s0 - kk;
+                next = strand ? s0 + kk : s1 - 1 - kk;
+            }
+        }
+        // Parts with several rows grow towards their first base while the group has
+        // more places than two rounds look at: a base costs about a third of a
+        // round, and leaves the copies of a repeat that differ there.
+        for (int step = 0; step < kExtend; step++) {
+            const uint32_t places = group_sum<G>(width);
+            const bool go = todo && bases && width > 2 && places > 2 * G;
+            if (!__any_sync(FULL, go)) break;
+            if (go) {
+                const uint32_t c = ((S.bases[next >> 4] >> (2 * (next & 15u))) & 3u) ^ (strand ? 3u : 0u);
+                lo = X.t[0].C1[c] + occ1(X.t[0], c, lo);
+                hi = X.t[0].C1[c] + occ1(X.t[0], c, hi);
+                width = hi > lo ? min(hi - lo, kWideRows) : 0u;
+                next += strand ? 1u : ~0u;
+                off--;
+                bases--;
+            }
+        }
+        // places of the group, shared out in order
+        uint32_t before = width;
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(FULL, before, o, G);
+            if (l >= static_cast<uint32_t>(o)) before += u;
+        }
+        uint32_t total = __shfl_sync(FULL, before, G - 1, G);
+        before -= width;
+        const bool again = todo && !stepping && b > 1 && total > kManyPlaces * G;
+        if (again) {
+            stepping = true;
+            total = 0;
+        } else if (todo && total > max_places) {
+            failed = true;
+            todo = false;
+        }
+        const uint32_t span = ps | (pe << 8) | (off << 16);
+        for (uint32_t c0 = 0; __any_sync(FULL, todo && c0 < total); c0 += G) {
+            const uint32_t c = c0 + l, have = min(S.count, static_cast<uint32_t>(E));
+            __syncwarp();  // before this round's lanes record targets
+            uint32_t o = 0;  // the lane whose part has place c: the last one that starts at or before it
+#pragma unroll
+            for (int step = G / 2; step; step >>= 1) {
+                const uint32_t u = __shfl_sync(FULL, before, static_cast<int>(o) + step, G);
+                if (u <= c) o += step;
+            }
+            const uint32_t orow = __shfl_sync(FULL, lo, static_cast<int>(o), G) +
+                                  (c - __shfl_sync(FULL, before, static_cast<int>(o), G));
+            const uint32_t ospan = __shfl_sync(FULL, span, static_cast<int>(o), G);
+            const uint32_t cs = o / kHalf;
+            const int qs = static_cast<int>(ospan & 0xFFu), qe = static_cast<int>((ospan >> 8) & 0xFFu);
+            bool live = todo && c < total;
+            long long d = 0;  // the diagonal: text position of pattern index 0
+            if (live) {
+                d = static_cast<long long>(__ldg(X.sa[0] + orow)) - static_cast<int>(ospan >> 16);
+                live = d >= -static_cast<int>(z) && d + m <= static_cast<long long>(n) + static_cast<int>(z);
+            }
+            const Pattern &P = S.pat[cs];
+            uint32_t mis[kPlaneWords];
+            uint32_t mm = 255;
+            if (live) {
+                mismatches(X.text, P, d, m, mis);
+                live = count_in(mis, qs, qe) == 0;  // else another part leads to what this diagonal has
+            }
+            // of the lanes on one diagonal the first looks on, for all their parts
+            const unsigned long long tag = live ? (static_cast<unsigned long long>(d + 16) << 8) |
+                                                      ((threadIdx.x & 31u) / G * 2 + cs)
+                                                : ~0ull - (threadIdx.x & 31u);
+            const unsigned same = __match_any_sync(FULL, tag);
+            const int first_end = static_cast<int>(__reduce_min_sync(same, static_cast<unsigned>(qe)));
+            const int last_start = static_cast<int>(__reduce_max_sync(same, static_cast<unsigned>(qs)));
+            live = live && static_cast<uint32_t>(__ffs(same) - 1) == (threadIdx.x & 31u);
+            if (live && d >= 0 && d + m <= static_cast<long long>(n)) {
+                mm = count_in(mis, 0, m);
+                if (p.seed_len && mm <= z) {
+                    const SeedZone Z = zone(cs);
+                    if (count_in(mis, Z.from, Z.to) > Z.most) mm = 255;
+                }
+            }
+            dmin = min(dmin, group_min<G>(mm));
+            if (!exhaustive) F = min(z, dmin + 1);
+            if (live && mm <= F) add_target(S, have, cs, d, static_cast<uint32_t>(m), mm, 0u);
+            // gapped targets: a diagonal whose prefix or suffix leaves differences for a
+            // gap is looked at by the whole group, one (gap, side) a lane
+            const uint32_t gmost = p.max_gapo ? min(F, p.max_gape + 1u) : 0u;
+            bool want = false;
+            if (live && gmost) {
+                const int f = static_cast<int>(F), gm = static_cast<int>(gmost), e = static_cast<int>(p.e);
+                want = (count_in(mis, 0, first_end) < F && gap_fits(X.text, P, d, m, mis, f, gm, e, false)) ||
+                       (count_in(mis, last_start, m) < F && gap_fits(X.text, P, d, m, mis, f, gm, e, true));
+            }
+            uint32_t dgap = 255;
+            for (unsigned left = __ballot_sync(FULL, want) & group_lanes; __any_sync(FULL, left != 0); left &= left - 1) {
+                const int src = left ? __ffs(left) - 1 : static_cast<int>(threadIdx.x & 31u);
+                uint32_t mo[kPlaneWords], md[kPlaneWords];
+#pragma unroll
+                for (int w = 0; w < kPlaneWords; w++) md[w] = __shfl_sync(FULL, mis[w], src);
+                const long long dd = __shfl_sync(FULL, d, src);
+                const uint32_t ds = __shfl_sync(FULL, cs, src);
+                const int fe = __shfl_sync(FULL, first_end, src), ls = __shfl_sync(FULL, last_start, src);
+                SeedZone Z = zone(ds);
+                for (uint32_t q = l; left && q < 4 * gmost; q += G) {
+                    const int g = static_cast<int>(q >> 2) + 1;
+                    const bool del = q & 1u, side = q & 2u;  // side 0: a part lies before the gap, 1: after it
+                    const uint32_t fixed = side ? count_in(md, ls, m) : count_in(md, 0, fe);
+                    const long long other = side == del ? dd - g : dd + g;
+                    const long long a = side ? other : dd;
+                    const int L = del ? m + g : m - g;
+                    int plo = del ? max(static_cast<int>(p.e), 1) : static_cast<int>(p.e);
+                    int phi = del ? m - plo : m - plo - g;
+                    if (side) phi = min(phi, ls - (del ? 0 : g));
+                    else plo = max(plo, fe);
+                    if (fixed + g > F || L < 1 || a < 0 || a + L > static_cast<long long>(n) || plo > phi) continue;
+                    mismatches(X.text, S.pat[ds], other, m, mo);
+                    if (side) {  // the prefix's mismatches, then the suffix's
+#pragma unroll
+                        for (int w = 0; w < kPlaneWords; w++) {
+                            const uint32_t t = mo[w];
+                            mo[w] = md[w];
+                            md[w] = t;
+                        }
+                    }
+                    const uint32_t f = best_gap(md, mo, m, g, del, plo, phi, F - g, Z);
+                    if (side) {
+#pragma unroll
+                        for (int w = 0; w < kPlaneWords; w++) md[w] = mo[w];
+                    }
+                    if (f != 0xFFFFFFFFu) {
+                        add_target(S, have, ds, a, static_cast<uint32_t>(L), f, static_cast<uint32_t>(g));
+                        dgap = min(dgap, f + static_cast<uint32_t>(g));
+                    }
+                }
+            }
+            dmin = min(dmin, group_min<G>(dgap));
+            if (!exhaustive) F = min(z, dmin + 1);
+            __syncwarp();
+        }
+        if (todo) {
+            if (S.count > static_cast<uint32_t>(E)) {
+                failed = true;
+                todo = false;
+            } else if (again) {
+                b = 1;
+            } else if (exhaustive || F <= b) {  // F = z while nothing is found
+                todo = false;
+            } else {
+                b = stepping ? min(F, b + 1) : F;
+            }
+        }
+    }
+
+    // ---- reduction of the targets: intervals, merged hits, strata, order
+    const uint32_t cnt = search && !failed ? min(S.count, static_cast<uint32_t>(E)) : 0u;
+    if (__all_sync(FULL, cnt <= 1u)) {  // the usual read: one target (its group's lanes 0), or none
+        if (l == 0 && search && !failed) {
+            const uint32_t key = cnt ? S.key[0] : 0u, a = S.start[0];
+            const bool any = cnt && key_diffs(key) <= F;
+            aln_read_result out;
+            out.c0 = any ? 1u : 0u;
+            out.c1 = 0;
+            out.n_hits = any ? 1 : 0;
+            out.flags = 0;
+            out.d_best = static_cast<uint8_t>(any ? key_diffs(key) : 255u);
+            out.best_score = static_cast<uint8_t>(SCORE ? (any ? min(key_score(p, key), 254u) : 255u) : 0u);
+            if (any) {
+                const uint32_t row = (key >> 31) ? row_of(X, 0, a) : row_of(X, 1, n - a - (key & 0xFFFFu));
+                put_hit(hits + static_cast<uint64_t>(r) * p.hit_cap, row, row, key);
+            }
+            res[r] = out;
+        } else if (l == 0 && answer) {
+            empty_result<SCORE>(res + r, flags);
+        }
+        return (search && !failed) || answer;
+    }
+    // targets above the final budget and second records leave; rows of the others
+    for (uint32_t e = l; e < cnt; e += G) {
+        const uint32_t key = S.key[e], a = S.start[e];
+        bool keep = key_diffs(key) <= F;
+        for (uint32_t j = 0; j < e && keep; j++) keep = !(S.start[j] == a && S.key[j] == key);
+        uint32_t row = 0xFFFFFFFFu;
+        if (keep) row = (key >> 31) ? row_of(X, 0, a) : row_of(X, 1, n - a - (key & 0xFFFFu));
+        S.row[e] = row;
+        S.end[e] = keep ? 1u : 0u;
+    }
+    __syncwarp();
+    // the first row of a run of equal targets stands for the run
+    for (uint32_t e = l; e < cnt; e += G) {
+        if (!S.end[e]) continue;
+        const uint32_t key = S.key[e], row = S.row[e], a = S.start[e];
+        uint32_t top = row;
+        bool first = true;
+        for (uint32_t j = 0; j < cnt && first; j++)
+            first = !(S.row[j] + 1u == row && S.row[j] != 0xFFFFFFFFu && S.key[j] == key &&
+                      same_text(X.text, S.start[j], a, key & 0xFFFFu));
+        bool more = first;
+        while (more) {
+            more = false;
+            for (uint32_t j = 0; j < cnt; j++)
+                if (S.row[j] == top + 1u && S.key[j] == key && S.row[j] != 0xFFFFFFFFu &&
+                    same_text(X.text, S.start[j], a, key & 0xFFFFu)) {
+                    top++;
+                    more = true;
+                    break;
+                }
+        }
+        S.end[e] = first ? top + 1u : 0u;  // no other lane reads it before the barrier
+    }
+    __syncwarp();
+    // hits of equal rows on a strand keep the least (score, witness)
+    uint32_t drop = 0, kept = 0, s1 = 0xFFFFFFFFu;
+    for (uint32_t e = l, i = 0; e < cnt; e += G, i++) {
+        const uint32_t key = S.key[e], row = S.row[e], end = S.end[e];
+        bool keep = end != 0u;
+        for (uint32_t j = 0; j < cnt && keep; j++)
+            if (j != e && S.row[j] == row && S.end[j] == end && (S.key[j] >> 31) == (key >> 31)) {
+                if (SCORE) {
+                    const uint32_t a = key_score(p, S.key[j]), c = key_score(p, key);
+                    keep = !(a < c || (a == c && S.key[j] < key));
+                } else {
+                    keep = !(S.key[j] < key);
+                }
+            }
+        if (!keep) drop |= 1u << i;
+        else if (SCORE) s1 = min(s1, key_score(p, key));
+        if (keep) kept++;
+    }
+    __syncwarp();
+    for (uint32_t e = l, i = 0; e < cnt; e += G, i++)
+        if ((drop >> i) & 1u) S.end[e] = 0u;
+    kept = group_sum<G>(kept);
+    if (kept > static_cast<uint32_t>(kCandCap)) failed = true;  // the tree search flags it
+    __syncwarp();
+    uint32_t best = 255, c0 = 0, c1 = 0, s2 = 0xFFFFFFFFu;
+    if (SCORE) {
+        s1 = group_min<G>(s1);
+        for (uint32_t e = l; e < cnt; e += G)
+            if (S.end[e]) {
+                const uint32_t sc = key_score(p, S.key[e]);
+                if (sc > s1) s2 = min(s2, sc);
+                else best = min(best, key_diffs(S.key[e]));
+            }
+        s2 = group_min<G>(s2);
+    } else {
+        for (uint32_t e = l; e < cnt; e += G)
+            if (S.end[e]) best = min(best, key_diffs(S.key[e]));
+    }
+    best = group_min<G>(best);
+    for (uint32_t e = l; e < cnt; e += G)
+        if (S.end[e]) {
+            const uint32_t w = S.end[e] - S.row[e];
+            const uint32_t v = SCORE ? key_score(p, S.key[e]) : key_diffs(S.key[e]);
+            if (v == (SCORE ? s1 : best)) c0 += w;
+            else if (v == (SCORE ? s2 : best + 1)) c1 += w;
+        }
+    c0 = group_sum<G>(c0);
+    c1 = group_sum<G>(c1);
+    const bool many = SCORE && p.max_best && c0 > p.max_best;
+    uint32_t listed = 0;
+    const bool write = search && !failed;
+    for (uint32_t e = l; e < cnt && write; e += G) {
+        if (!S.end[e]) continue;
+        const uint32_t key = S.key[e], row = S.row[e], end = S.end[e];
+        const uint32_t v = SCORE ? key_score(p, key) : key_diffs(key);
+        if (SCORE && v != s1 && (many || v != s2)) continue;
+        listed++;
+        uint32_t rank = 0;  // hits before it in the order (diffs or score, strand, k, l)
+        for (uint32_t j = 0; j < cnt; j++) {
+            if (!S.end[j] || j == e) continue;
+            const uint32_t kj = S.key[j], vj = SCORE ? key_score(p, kj) : key_diffs(kj);
+            const uint32_t oj = (vj << 1) | (kj >> 31), oe = (v << 1) | (key >> 31);
+            rank += oj < oe || (oj == oe && (S.row[j] < row || (S.row[j] == row && S.end[j] < end))) ? 1u : 0u;
+        }
+        if (rank < p.hit_cap) {
+            put_hit(hits + static_cast<uint64_t>(r) * p.hit_cap + rank, row, end - 1u, key);
+        }
+    }
+    listed = group_sum<G>(listed);
+    if (answer && l == 0) empty_result<SCORE>(res + r, flags);
+    if (write && l == 0) {
+        aln_read_result out;
+        const bool any = listed > 0;
+        if (many) flags |= ALN_FLAG_MANY_BEST;
+        if (listed > p.hit_cap) flags |= ALN_FLAG_HIT_OVERFLOW;
+        out.c0 = any ? c0 : 0u;
+        out.c1 = any ? c1 : 0u;
+        out.n_hits = static_cast<uint8_t>(min(listed, p.hit_cap));
+        out.d_best = static_cast<uint8_t>(any ? best : 255u);
+        out.best_score = static_cast<uint8_t>(SCORE ? (any ? min(s1, 254u) : 255u) : 0u);
+        out.flags = static_cast<uint8_t>(flags);
+        res[r] = out;
+    }
+    return write || answer;
+}
+
+}  // namespace aln
