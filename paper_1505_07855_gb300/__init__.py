@@ -298,8 +298,27 @@ class Aligner:
         if check_status:
             self.check_status()
         r = res.cpu().numpy().view(RES_DTYPE)[:n]
-        h = hits.cpu().numpy().view(HIT_DTYPE)[:n * params.hit_cap].reshape(n, params.hit_cap)
-        return r, h
+        return r, self._hits_to_host(res, hits, r, params.hit_cap)
+
+    def _hits_to_host(self, res, hits, r, cap: int):
+        """hits[n, cap] of a finished search on the host; slots past a read's n_hits
+        are undefined.  A read usually has one hit of its cap slots: where at most
+        half of the slots are written, they are compacted on the device and put
+        in their places here (100 000 reads of 32 slots: 1.6 MB copied, not 51)."""
+        t, n = self.torch, r.size
+        total = int(r["n_hits"].sum(dtype=np.int64))
+        if n == 0 or 2 * total > n * cap or n * cap >= 1 << 32:
+            return hits.cpu().numpy().view(HIT_DTYPE)[:n * cap].reshape(n, cap)
+        h = np.empty((n, cap), HIT_DTYPE)
+        if total:
+            off = t.empty(n + 1, dtype=t.int32, device=self.dev)
+            dense = t.empty(total * HIT_DTYPE.itemsize, dtype=t.uint8, device=self.dev)
+            self.compact(res, hits, n, cap, off, dense, self.compact_scratch(n), t.cuda.current_stream(self.dev))
+            count = r["n_hits"].astype(np.int64)
+            at = np.repeat(np.arange(n, dtype=np.int64) * cap - (np.cumsum(count) - count), count)
+            at += np.arange(total, dtype=np.int64)
+            h.reshape(-1)[at] = dense.cpu().numpy().view(HIT_DTYPE)
+        return h
 
     def compact(self, res, hits, n: int, hit_cap: int, offsets, dense, scratch, stream=None) -> None:
         """aln_compact_hits on device buffers: offsets (n + 1 uint32), dense hits

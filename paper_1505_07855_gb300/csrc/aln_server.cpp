@@ -26,6 +26,7 @@
 
 #include "aln_gb300.h"
 #include "aln_internal.h"
+#include "aln_pack.h"
 
 namespace {
 
@@ -134,6 +135,7 @@ static uint64_t slot_bytes(const aln_server_config &c) {
 static uint64_t pack_slot(Slot &s, const aln_server_config &c) {
     uint64_t j = 0;
     uint32_t r = 0;
+    aln::Packer P(s.h_bases, s.h_nmask, 0);
     for (Chunk &ch : s.chunks) {
         ch.slot_first = r;
         const Request &q = *ch.req;
@@ -141,20 +143,13 @@ static uint64_t pack_slot(Slot &s, const aln_server_config &c) {
             s.h_off[r] = j;
             s.h_len[r] = q.len[t];
             s.h_z[r] = q.z.empty() ? c.params.z : q.z[t];
-            const uint8_t *cd = q.codes.data() + q.off[t];
-            const uint32_t L = q.len[t];
-            for (uint32_t u = 0; u < L; u++, j++) {
-                if ((j & 15) == 0) s.h_bases[j >> 4] = 0;
-                if ((j & 31) == 0) s.h_nmask[j >> 5] = 0;
-                uint32_t b = cd[u];
-                if (b > 3) {
-                    s.h_nmask[j >> 5] |= 1u << (j & 31);
-                    b = 0;
-                }
-                s.h_bases[j >> 4] |= b << (2 * (j & 15));
-            }
+            P.read(q.codes.data() + q.off[t], q.len[t]);
+            j += q.len[t];
         }
     }
+    if (j % 16) s.h_bases[j / 16] = 0;
+    if (j % 32) s.h_nmask[j / 32] = 0;
+    P.finish();
     s.n_reads = r;
     return j;
 }

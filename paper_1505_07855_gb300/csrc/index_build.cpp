@@ -18,11 +18,13 @@
 #include <atomic>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <fstream>
 #include <new>
 #include <thread>
 
 #include "aln_internal.h"
+#include "aln_pack.h"
 
 namespace aln {
 
@@ -457,22 +459,37 @@ extern "C" int aln_pack_reads(const uint8_t *codes, const uint64_t *code_offset,
     if (n_reads && (!codes || !code_offset || !len || !bases_out || !nmask_out || !offset_out))
         return fail(ALN_EINVAL, "aln_pack_reads: null argument");
     uint64_t total = 0;
-    for (uint32_t r = 0; r < n_reads; r++) total += len[r];
-    std::memset(bases_out, 0, ((total + 15) / 16) * 4);
-    std::memset(nmask_out, 0, ((total + 31) / 32) * 4);
-    uint64_t j = 0;
     for (uint32_t r = 0; r < n_reads; r++) {
-        offset_out[r] = j;
-        const uint8_t *c = codes + code_offset[r];
-        for (uint32_t t = 0; t < len[r]; t++, j++) {
-            uint32_t b = c[t];
-            if (b > 3) {
-                nmask_out[j / 32] |= 1u << (j % 32);
-                b = 0;
-            }
-            bases_out[j / 16] |= b << (2 * (j % 16));
-        }
+        offset_out[r] = total;
+        total += len[r];
     }
+    if (total == 0) return ALN_OK;
+    // ranges of reads, one a thread (a range of 2^18 bases takes about 0.1 ms on
+    // one core); a range's first and last words may be shared with its neighbours
+    const uint64_t most = std::min<uint64_t>(16, static_cast<uint64_t>(resolve_threads(0)));
+    const uint64_t ranges = std::max<uint64_t>(1, std::min<uint64_t>({most, total >> 18, n_reads}));
+    auto first_read = [&](uint64_t i) { return static_cast<uint32_t>(n_reads * i / ranges); };
+    for (uint64_t i = 0; i <= ranges; i++) {
+        const uint64_t at = i < ranges ? std::min(offset_out[first_read(i)], total - 1) : total - 1;
+        bases_out[at / 16] = 0;
+        nmask_out[at / 32] = 0;
+    }
+    auto pack = [&](uint64_t i) {
+        const uint32_t r0 = first_read(i), r1 = first_read(i + 1);
+        aln::Packer P(bases_out, nmask_out, offset_out[r0]);
+        for (uint32_t r = r0; r < r1; r++) P.read(codes + code_offset[r], len[r]);
+        P.finish();
+    };
+    std::vector<std::thread> th;
+    uint64_t started = 1;
+    try {
+        th.reserve(ranges);
+        for (; started < ranges; started++) th.emplace_back(pack, started);
+    } catch (const std::exception &) {  // no thread to be had: the rest is packed here
+    }
+    pack(0);
+    for (uint64_t i = started; i < ranges; i++) pack(i);
+    for (auto &t : th) t.join();
     return ALN_OK;
 }
 
