@@ -12,6 +12,7 @@
 // is N, 1 insertion, 4 deletions), and only when no entry with d+1 is on the
 // stack.  Hence at most 1 + 9*B entries for budget B; the capacity is chosen
 // from z so the overflow flag cannot be raised.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <string>
@@ -50,7 +51,7 @@ constexpr uint32_t kPlainReads = kThreads / 4;    // reads of a seeded block
 constexpr uint32_t kPlainTargets = 32, kPlainPlaces = 2048;
 
 template <int STACK_CAP>
-__global__ void __launch_bounds__(kThreads) aln_plain_kernel(DIndex X, ReadBatch rb, uint32_t n_reads, SearchParams p,
+__global__ void __launch_bounds__(kThreads) aln_plain_kernel(const __grid_constant__ DIndex X, ReadBatch rb, uint32_t n_reads, const __grid_constant__ SearchParams p,
                                                              aln_read_result *res, aln_hit *hits, bool seeded) {
     __shared__ union {
         SeedRead<kPlainTargets> read[kThreads / kPlainLanes];
@@ -95,6 +96,7 @@ __global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_persi
                                                                   SearchParams p, aln_read_result *res,
                                                                   aln_hit *hits, uint32_t *queue,
                                                                   const uint32_t *order, const uint2 *dbp) {
+    cudaGridDependencySynchronize();
     // after a seed search that left no read, the queue starts at its end
     if (__all_sync(0xFFFFFFFFu, *reinterpret_cast<volatile uint32_t *>(queue) >= n_reads)) return;
     __shared__ uint32_t s_bases[kReadWords * kThreads];
@@ -267,10 +269,7 @@ __device__ bool heavy_insert(const HeavyCtx &H, uint32_t hid, uint32_t s, uint32
 // the lower bound admits as a task, for the deepening pass the read was in when
 // it was handed over (R->B, written by its lane).  Each pass starts from the
 // root with no candidates, so the passes before it need not be searched again.
-__global__ void aln_heavy_start_kernel(SearchParams p, const uint2 *dbp, uint32_t n_text) {
-    const HeavyCtx H = p.heavy;
-    const uint32_t hid = blockIdx.x;
-    if (hid >= min(H.hdr->n_heavy, kHeavyReads)) return;
+__device__ void heavy_start_one(const HeavyCtx &H, uint32_t hid, const uint2 *dbp, uint32_t n_text) {
     HeavySlot *T = H.slots + static_cast<uint64_t>(hid) * 2 * kHeavySlots;
     for (uint32_t j = threadIdx.x; j < 2 * kHeavySlots; j += blockDim.x) {
         T[j].id = 0ull;
@@ -287,6 +286,19 @@ __global__ void aln_heavy_start_kernel(SearchParams p, const uint2 *dbp, uint32_
         const uint4 root = make_uint4(0, n_text + 1, pack_info(0, 0, 0, 0, 0, 0, OP_M), 0);
         if (d0 <= R->B) heavy_push(H, root, hid, 0);
         if (d1 <= R->B) heavy_push(H, root, hid, 1);
+    }
+}
+
+// Blocks of the start and decide kernels: a call without heavy reads, the usual
+// one, only pays for launching them (2048 blocks, one a possible read: 3.3 us).
+constexpr uint32_t kHeavyBlocks = 152;
+
+__global__ void aln_heavy_start_kernel(SearchParams p, const uint2 *dbp, uint32_t n_text) {
+    cudaGridDependencySynchronize();
+    const uint32_t n = min(p.heavy.hdr->n_heavy, kHeavyReads);
+    for (uint32_t hid = blockIdx.x; hid < n; hid += gridDim.x) {
+        heavy_start_one(p.heavy, hid, dbp, n_text);
+        __syncthreads();
     }
 }
 
@@ -529,6 +541,7 @@ template <int STACK_CAP, bool SCORE>
 __global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_heavy_pass_kernel(DIndex X, ReadBatch rb,
                                                                                            SearchParams p,
                                                                                            const uint2 *dbp) {
+    cudaGridDependencySynchronize();
     heavy_pass<STACK_CAP, SCORE>(X, rb, p, dbp);
 }
 
@@ -622,11 +635,9 @@ __device__ void heavy_write_score(const SearchParams &p, const HeavySlot *T, con
 
 // One block per handed-over read after a pass: the iterative deepening rule on
 // its table; the result, or the next pass's budget, cleared tables and roots.
-__global__ void aln_heavy_decide_kernel(SearchParams p, const uint2 *dbp, uint32_t n_text, aln_read_result *res,
-                                        aln_hit *hits, int last) {
+__device__ void heavy_decide_one(const SearchParams &p, uint32_t hid, const uint2 *dbp, uint32_t n_text,
+                                 aln_read_result *res, aln_hit *hits, int last) {
     const HeavyCtx H = p.heavy;
-    const uint32_t hid = blockIdx.x;
-    if (hid >= min(H.hdr->n_heavy, kHeavyReads)) return;
     HeavyRead *R = H.reads + hid;
     if (R->state != 0) return;
     HeavySlot *T = H.slots + static_cast<uint64_t>(hid) * 2 * kHeavySlots;
@@ -767,6 +778,41 @@ __global__ void aln_heavy_decide_kernel(SearchParams p, const uint2 *dbp, uint32
     R->state = 1;
 }
 
+__global__ void aln_heavy_decide_kernel(SearchParams p, const uint2 *dbp, uint32_t n_text, aln_read_result *res,
+                                        aln_hit *hits, int last) {
+    cudaGridDependencySynchronize();
+    const uint32_t n = min(p.heavy.hdr->n_heavy, kHeavyReads);
+    for (uint32_t hid = blockIdx.x; hid < n; hid += gridDim.x) {
+        heavy_decide_one(p, hid, dbp, n_text, res, hits, last);
+        __syncthreads();
+    }
+}
+
+// The whole phase in one cooperative launch, a grid barrier where the kernels
+// above follow each other: for a call of at most kHeavyReads reads, whose time is
+// that of its launches when, as usual, no read is heavy (a call of 64 reads
+// launched 11 kernels to find that out).
+template <int STACK_CAP, bool SCORE>
+__global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_heavy_all_kernel(
+    DIndex X, ReadBatch rb, SearchParams p, const uint2 *dbp, aln_read_result *res, aln_hit *hits) {
+    const uint32_t n = min(p.heavy.hdr->n_heavy, kHeavyReads);  // no kernel of the phase changes it
+    if (n == 0) return;
+    const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+    for (uint32_t hid = blockIdx.x; hid < n; hid += gridDim.x) {
+        heavy_start_one(p.heavy, hid, dbp, X.t[0].n);
+        __syncthreads();
+    }
+    for (uint32_t pass = 0; pass < kHeavyPasses; pass++) {
+        grid.sync();
+        heavy_pass<STACK_CAP, SCORE>(X, rb, p, dbp);
+        grid.sync();
+        for (uint32_t hid = blockIdx.x; hid < n; hid += gridDim.x) {
+            heavy_decide_one(p, hid, dbp, X.t[0].n, res, hits, pass + 1 == kHeavyPasses ? 1 : 0);
+            __syncthreads();
+        }
+    }
+}
+
 // ---------------------------------------------------------------- end of the heavy phase
 
 #ifdef ALN_STATS
@@ -822,11 +868,15 @@ struct SeedCounts {          // in the scratch's first words, cleared before the
 };
 
 // Room for targets and places to look at, first for a read's 8 or 16 lanes: past
-// that the other reads of the warp wait for it, so it goes to a warp of its own.
+// that the other reads of the warp wait for it, so it goes to a warp of its own
+// (300 000 mates on 3.1 Gbp: 8.4 / 7.15 / 6.2 ms with 1024 / 256 / 64 places).
 // There, kCandCap targets are what the tree search keeps, and 16384 places are half
 // a millisecond of a warp, about what the tree search of such a read costs.
 constexpr uint32_t kSeedTargets = 32;
-constexpr uint32_t kSeedPlaces = 256;
+#ifndef ALN_SEED_PLACES
+#define ALN_SEED_PLACES 64
+#endif
+constexpr uint32_t kSeedPlaces = ALN_SEED_PLACES;
 constexpr uint32_t kWidePlaces = 16384;
 
 // Resident blocks per SM: 4 / 5 / 6 take 4.2 / 3.97 / 3.89 ms for 1 M reads of 100
@@ -840,12 +890,15 @@ constexpr uint32_t kWidePlaces = 16384;
 #endif
 
 template <int G, bool SCORE>
-__global__ void __launch_bounds__(kThreads, ALN_SEED_MIN_BLOCKS) aln_seed_kernel(DIndex X, ReadBatch rb, uint32_t n, SearchParams p,
+__global__ void __launch_bounds__(kThreads, ALN_SEED_MIN_BLOCKS) aln_seed_kernel(const __grid_constant__ DIndex X, ReadBatch rb, uint32_t n, const __grid_constant__ SearchParams p,
                                                             aln_read_result *res, aln_hit *hits, SeedCounts *counts,
                                                             uint32_t *wide) {
     __shared__ SeedRead<kSeedTargets> s_read[kThreads / G];
-    if (blockIdx.x == 0 && p.heavy.hdr && threadIdx.x < sizeof(HeavyHdr) / 4)  // what the heavy phase counts in
-        reinterpret_cast<uint32_t *>(p.heavy.hdr)[threadIdx.x] = 0;
+    if (blockIdx.x == 0) {  // what the later kernels report and count in
+        if (p.status && threadIdx.x == 0) *p.status = 0;
+        if (p.heavy.hdr && threadIdx.x < sizeof(HeavyHdr) / 4)
+            reinterpret_cast<uint32_t *>(p.heavy.hdr)[threadIdx.x] = 0;
+    }
     const uint64_t r = (static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x) / G;
     const bool active = r < n;
     const bool done = seed_search<G, kSeedTargets, SCORE>(X, rb, p, s_read[threadIdx.x / G], static_cast<uint32_t>(r),
@@ -854,11 +907,12 @@ __global__ void __launch_bounds__(kThreads, ALN_SEED_MIN_BLOCKS) aln_seed_kernel
 }
 
 template <bool SCORE>
-__global__ void __launch_bounds__(kThreads, ALN_WIDE_MIN_BLOCKS) aln_seed_wide_kernel(DIndex X, ReadBatch rb, SearchParams p,
+__global__ void __launch_bounds__(kThreads, ALN_WIDE_MIN_BLOCKS) aln_seed_wide_kernel(const __grid_constant__ DIndex X, ReadBatch rb, const __grid_constant__ SearchParams p,
                                                                  aln_read_result *res, aln_hit *hits,
                                                                  SeedCounts *counts, const uint32_t *wide,
                                                                  uint32_t *order_end) {
     __shared__ SeedRead<kCandCap> s_read[kThreads / 32];
+    cudaGridDependencySynchronize();
     const uint32_t lane = threadIdx.x & 31u, n = counts->wide;
     for (;;) {
         uint32_t i = 0;
@@ -878,6 +932,7 @@ __global__ void __launch_bounds__(kThreads) aln_dscan_list_kernel(DIndex X, Read
                                                                   uint2 *dbp) {
     __shared__ uint32_t s_bases[kReadWords * kThreads];
     __shared__ uint32_t s_nmask[kMaskWords * kThreads];
+    cudaGridDependencySynchronize();
     const uint32_t n = counts->rest;
     if (blockIdx.x == 0 && threadIdx.x == 0) *queue = n_reads - n;
     if (n == 0) return;
@@ -936,6 +991,34 @@ __global__ void aln_order_scatter_kernel(const uint2 *dbp, uint32_t n, const uin
     }
 }
 
+// A launch that may be prepared while the kernel before it on the stream drains
+// (the kernel waits for it at its start): most of a call's kernels find nothing
+// to do, and a call's time is then that of its launches (64 reads: 77 -> 58 us
+// with the heavy phase in one launch; 30 000 reads: 195 -> 162 us).
+template <class... Params, class... Args>
+static cudaError_t launch_after(void (*kernel)(Params...), unsigned blocks, cudaStream_t st, const SearchParams *window,
+                                Args &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (window && window->window_base && window->window_bytes) {  // prefix-trie tables held in L2's persisting set
+        attr[1].id = cudaLaunchAttributeAccessPolicyWindow;
+        attr[1].val.accessPolicyWindow.base_ptr = window->window_base;
+        attr[1].val.accessPolicyWindow.num_bytes = window->window_bytes;
+        attr[1].val.accessPolicyWindow.hitRatio = window->window_hit_ratio;
+        attr[1].val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
+        attr[1].val.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
+        cfg.numAttrs = 2;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 int stack_cap_for(uint32_t z) { return z <= 2 ? 19 : (z <= 4 ? 37 : 64); }
 HeavyCtx heavy_layout(void *scratch, uint32_t n);
 
@@ -978,9 +1061,11 @@ static cudaError_t launch_cap(const DIndex &X, const ReadBatch &rb, uint32_t n, 
                 aln_seed_kernel<16, SCORE><<<static_cast<unsigned>((16ull * n + kThreads - 1) / kThreads), kThreads, 0, st>>>(
                     X, rb, n, pp, res, hits, counts, wide);
             const uint32_t wb = min((n + 3u) / 4u, static_cast<uint32_t>(sms) * 6u);
-            aln_seed_wide_kernel<SCORE><<<wb, kThreads, 0, st>>>(X, rb, pp, res, hits, counts, wide, order + n);
+            cudaError_t e = launch_after(aln_seed_wide_kernel<SCORE>, wb, st, nullptr, X, rb, pp, res, hits, counts, wide,
+                                         order + n);
             const uint32_t db = min(static_cast<uint32_t>((2ull * n + kThreads - 1) / kThreads), static_cast<uint32_t>(sms) * 8u);
-            aln_dscan_list_kernel<<<db, kThreads, 0, st>>>(X, rb, pp, n, order, counts, queue, dbp);
+            if (e == cudaSuccess) e = launch_after(aln_dscan_list_kernel, db, st, nullptr, X, rb, pp, n, order, counts, queue, dbp);
+            if (e != cudaSuccess) return e;
         } else {
             cudaMemsetAsync(queue, 0, sizeof(uint32_t), st);
         }
@@ -1000,40 +1085,36 @@ static cudaError_t launch_cap(const DIndex &X, const ReadBatch &rb, uint32_t n, 
             aln_order_count_kernel<<<ob, 256, 0, st>>>(dbp, n, counts);
             aln_order_scatter_kernel<<<ob, 256, 0, st>>>(dbp, n, counts, cursor, order);
         }
-        const SearchParams &p1 = pp;
-        if (p.window_base && p.window_bytes) {  // prefix-trie tables held in L2's persisting set
+        cudaError_t e = launch_after(aln_persistent_kernel<CAP, SMEM, SCORE>, blocks, st, &p, X, rb, n, pp, res, hits, queue,
+                                     order, dbp);
+        if (e != cudaSuccess) return e;
+        if (pp.heavy.hdr && seeded && n <= kHeavyReads) {
+            int hb = 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&hb, aln_heavy_all_kernel<CAP, SCORE>, kThreads, 0);
             cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3(blocks);
+            cfg.gridDim = dim3(min(static_cast<unsigned>(sms * (hb > 0 ? hb : 1)), kHeavyPool / (2u * kThreads)));
             cfg.blockDim = dim3(kThreads);
             cfg.stream = st;
             cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeAccessPolicyWindow;
-            attr[0].val.accessPolicyWindow.base_ptr = p.window_base;
-            attr[0].val.accessPolicyWindow.num_bytes = p.window_bytes;
-            attr[0].val.accessPolicyWindow.hitRatio = p.window_hit_ratio;
-            attr[0].val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
-            attr[0].val.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
+            attr[0].id = cudaLaunchAttributeCooperative;
+            attr[0].val.cooperative = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            const cudaError_t e = cudaLaunchKernelEx(&cfg, aln_persistent_kernel<CAP, SMEM, SCORE>, X, rb, n, p1, res, hits,
-                                                     queue, static_cast<const uint32_t *>(order),
-                                                     static_cast<const uint2 *>(dbp));
+            e = cudaLaunchKernelEx(&cfg, aln_heavy_all_kernel<CAP, SCORE>, X, rb, pp, static_cast<const uint2 *>(dbp), res, hits);
             if (e != cudaSuccess) return e;
-        } else {
-            aln_persistent_kernel<CAP, SMEM, SCORE><<<blocks, kThreads, 0, st>>>(X, rb, n, p1, res, hits, queue, order,
-                                                                                dbp);
-        }
-        if (pp.heavy.hdr) {  // the reads handed over, one deepening pass per launch over the whole GPU
+        } else if (pp.heavy.hdr) {  // the reads handed over, one deepening pass per launch over the whole GPU
             int hb = 0;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&hb, aln_heavy_pass_kernel<CAP, SCORE>, kThreads, 0);
             // the ring holds at most 2 entries per thread of the grid (the pass kernel's low-water mark)
             const unsigned hgrid = min(static_cast<unsigned>(sms * (hb > 0 ? hb : 1)), kHeavyPool / (2u * kThreads));
-            aln_heavy_start_kernel<<<kHeavyReads, 128, 0, st>>>(pp, dbp, X.t[0].n);
-            for (uint32_t pass = 0; pass < kHeavyPasses; pass++) {
-                aln_heavy_pass_kernel<CAP, SCORE><<<hgrid, kThreads, 0, st>>>(X, rb, pp, dbp);
-                aln_heavy_decide_kernel<<<kHeavyReads, 128, 0, st>>>(pp, dbp, X.t[0].n, res, hits,
-                                                                    pass + 1 == kHeavyPasses ? 1 : 0);
+            e = launch_after(aln_heavy_start_kernel, kHeavyBlocks, st, nullptr, pp, dbp, X.t[0].n);
+            for (uint32_t pass = 0; pass < kHeavyPasses && e == cudaSuccess; pass++) {
+                e = launch_after(aln_heavy_pass_kernel<CAP, SCORE>, hgrid, st, nullptr, X, rb, pp, dbp);
+                if (e == cudaSuccess)
+                    e = launch_after(aln_heavy_decide_kernel, kHeavyBlocks, st, nullptr, pp, dbp, X.t[0].n, res, hits,
+                                     pass + 1 == kHeavyPasses ? 1 : 0);
             }
+            if (e != cudaSuccess) return e;
         }
     }
     return cudaGetLastError();
@@ -1104,7 +1185,8 @@ static cudaError_t launch_smem(const DIndex &X, const ReadBatch &rb, uint32_t n,
 cudaError_t launch_search(const DIndex &X, const ReadBatch &rb, uint32_t n, const SearchParams &p,
                           aln_read_result *res, aln_hit *hits, uint32_t mode, uint32_t *queue, void *scratch,
                           cudaStream_t st) {
-    if (p.status) {
+    const bool seeds = mode != ALN_MODE_PLAIN && n && scratch && seed_supported(X, p);  // its first kernel clears the status
+    if (p.status && !seeds) {
         const cudaError_t e = cudaMemsetAsync(p.status, 0, sizeof(uint32_t), st);
         if (e != cudaSuccess) return e;
     }
