@@ -1,7 +1,9 @@
 // Device-wide scan (sum or max) of 32-bit words, written for this library:
 // tiles of 4096 words, each reduced by one block, the tile reductions scanned
 // recursively, then every tile scanned with its prefix.  Used by the GPU index
-// builder and by the hit compaction.
+// builder and by the hit compaction.  The elements come from a functor and the
+// results go to one (element index, result), so that a pass that only prepares a
+// scan's input, or only uses its output, is part of the scan.
 #pragma once
 
 #include <cstdint>
@@ -55,15 +57,24 @@ __device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t *warp_t
     return mine;
 }
 
-template <class Op>
-__global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(const uint32_t *in, uint64_t n, uint32_t *partial, Op op) {
+struct LoadWord {
+    const uint32_t *in;
+    __device__ __forceinline__ uint32_t operator()(uint64_t j) const { return in[j]; }
+};
+struct StoreWord {
+    uint32_t *out;
+    __device__ __forceinline__ void operator()(uint64_t j, uint32_t v) const { out[j] = v; }
+};
+
+template <class Op, class Load>
+__global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(Load in, uint64_t n, uint32_t *partial, Op op) {
     __shared__ uint32_t wt[32];
     const uint64_t base = static_cast<uint64_t>(blockIdx.x) * kScanTile;
     uint32_t acc = 0;
 #pragma unroll
     for (int i = 0; i < kScanItems; i++) {
         const uint64_t j = base + static_cast<uint64_t>(i) * kScanThreads + threadIdx.x;
-        if (j < n) acc = op(acc, in[j]);
+        if (j < n) acc = op(acc, in(j));
     }
     uint32_t total = 0;
     block_exclusive(acc, wt, &total, op);
@@ -73,9 +84,9 @@ __global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(const uint32_
 // Scan of one tile: coalesced load into shared memory, 8 consecutive items per
 // thread, block scan of the thread sums, coalesced store.  prefix: the
 // exclusive scan of the tile reductions (nullptr: a single tile).
-template <class Op>
-__global__ void __launch_bounds__(kScanThreads) scan_tile_kernel(const uint32_t *in, uint32_t *out, uint64_t n,
-                                                                 const uint32_t *prefix, bool inclusive, Op op) {
+template <class Op, class Load, class Store>
+__global__ void __launch_bounds__(kScanThreads) scan_tile_kernel(Load in, Store out, uint64_t n, const uint32_t *prefix,
+                                                                 bool inclusive, Op op) {
     __shared__ uint32_t s[kScanTile];
     __shared__ uint32_t wt[32];
     const uint64_t base = static_cast<uint64_t>(blockIdx.x) * kScanTile;
@@ -83,7 +94,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_tile_kernel(const uint32_t 
     for (int i = 0; i < kScanItems; i++) {
         const uint32_t t = i * kScanThreads + threadIdx.x;
         const uint64_t j = base + t;
-        s[t] = j < n ? in[j] : 0u;
+        s[t] = j < n ? in(j) : 0u;
     }
     __syncthreads();
     uint32_t v[kScanItems];
@@ -106,7 +117,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_tile_kernel(const uint32_t 
     for (int i = 0; i < kScanItems; i++) {
         const uint32_t t = i * kScanThreads + threadIdx.x;
         const uint64_t j = base + t;
-        if (j < n) out[j] = s[t];
+        if (j < n) out(j, s[t]);
     }
 }
 
@@ -117,20 +128,27 @@ inline uint64_t scan_temp_words(uint64_t n) {
     return w + 2;
 }
 
-// out = scan of in (in == out allowed), exclusive or inclusive, sum or max.
-template <class Op>
-inline void device_scan(const uint32_t *in, uint32_t *out, uint64_t n, bool inclusive, uint32_t *temp, cudaStream_t st,
-                 Op op) {
+// out(j, r_j) for the scan r of in(0 .. n-1), exclusive or inclusive, sum or max.
+// Each element is read twice, the second time by the thread block that stores it.
+template <class Op, class Load, class Store>
+inline void device_scan_with(Load in, Store out, uint64_t n, bool inclusive, uint32_t *temp, cudaStream_t st, Op op) {
     if (n == 0) return;
     const uint64_t tiles = (n + kScanTile - 1) / kScanTile;
     if (tiles == 1) {
-        scan_tile_kernel<Op><<<1, kScanThreads, 0, st>>>(in, out, n, nullptr, inclusive, op);
+        scan_tile_kernel<Op, Load, Store><<<1, kScanThreads, 0, st>>>(in, out, n, nullptr, inclusive, op);
         return;
     }
     uint32_t *partial = temp, *pre = temp + tiles;
-    scan_reduce_kernel<Op><<<static_cast<unsigned>(tiles), kScanThreads, 0, st>>>(in, n, partial, op);
-    device_scan(partial, pre, tiles, false, temp + 2 * tiles, st, op);
-    scan_tile_kernel<Op><<<static_cast<unsigned>(tiles), kScanThreads, 0, st>>>(in, out, n, pre, inclusive, op);
+    scan_reduce_kernel<Op, Load><<<static_cast<unsigned>(tiles), kScanThreads, 0, st>>>(in, n, partial, op);
+    device_scan_with(LoadWord{partial}, StoreWord{pre}, tiles, false, temp + 2 * tiles, st, op);
+    scan_tile_kernel<Op, Load, Store><<<static_cast<unsigned>(tiles), kScanThreads, 0, st>>>(in, out, n, pre, inclusive, op);
+}
+
+// out = scan of in (in == out allowed).
+template <class Op>
+inline void device_scan(const uint32_t *in, uint32_t *out, uint64_t n, bool inclusive, uint32_t *temp, cudaStream_t st,
+                        Op op) {
+    device_scan_with(LoadWord{in}, StoreWord{out}, n, inclusive, temp, st, op);
 }
 
 }  // namespace

@@ -38,13 +38,17 @@ using scan::OpAdd;
 using scan::OpMax;
 using scan::block_exclusive;
 using scan::device_scan;
+using scan::device_scan_with;
 using scan::scan_temp_words;
 
 // ------------------------------------------------------------------ radix sort
 
 constexpr int kRsThreads = 256;
 constexpr int kRsWarps = kRsThreads / 32;
-constexpr int kRsRounds = 16;                                   // rounds of 32 items per warp
+#ifndef ALN_RS_ROUNDS
+#define ALN_RS_ROUNDS 16
+#endif
+constexpr int kRsRounds = ALN_RS_ROUNDS;                                   // rounds of 32 items per warp
 constexpr uint32_t kRsTile = kRsThreads * kRsRounds;            // 4096 items per tile
 constexpr int kRsBins = 256;
 template <class K>
@@ -219,51 +223,52 @@ __device__ __forceinline__ bool run_starts(const K *key, const uint32_t *val, ui
     return i == 0 || key[i] != key[i - 1] || (val && n - val[i - 1] < first);
 }
 
-// head[i] = i where key[i] starts a run of equal keys, else 0 (max-scan input).
+// After a sort of the m active rows by key, two scans place the suffixes.  The
+// first, a running maximum of the rows that start a run, gives each suffix the
+// first row of its run: the suffix order goes back into sa at the rows that the
+// active set occupies, and that first row becomes the suffix's rank.
+// A == nullptr: the active set is every row.
 template <class K>
-__global__ void run_head_kernel(const K *key, const uint32_t *val, uint64_t n, uint64_t m, uint32_t *head) {
-    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < m;
-         i += static_cast<uint64_t>(gridDim.x) * blockDim.x)
-        head[i] = run_starts(key, val, n, kFirst<K>, i) ? static_cast<uint32_t>(i) : 0u;
-}
-
-// After a sort of the active rows: the suffix order goes back into sa at the
-// rows the active set occupies, and each suffix's rank becomes the row of the
-// first member of its new run.  A == nullptr: the active set is every row.
-__global__ void place_rank_kernel(const uint32_t *A, const uint32_t *v, const uint32_t *start, uint64_t m,
-                                  uint32_t *sa, uint32_t *rank) {
-    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < m;
-         i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        const uint32_t row = A ? A[i] : static_cast<uint32_t>(i);
+struct RunHead {
+    const K *key;
+    const uint32_t *val;
+    uint64_t n;
+    __device__ __forceinline__ uint32_t operator()(uint64_t i) const {
+        return run_starts(key, val, n, kFirst<K>, i) ? static_cast<uint32_t>(i) : 0u;
+    }
+};
+struct PlaceRank {
+    const uint32_t *A, *v;
+    uint32_t *sa, *rank;
+    __device__ __forceinline__ void operator()(uint64_t i, uint32_t start) const {
         const uint32_t s = v[i];
-        sa[row] = s;
-        rank[s] = A ? A[start[i]] : start[i];
+        sa[A ? A[i] : static_cast<uint32_t>(i)] = s;
+        rank[s] = A ? A[start] : start;
     }
-}
+};
 
-// active[i] = 1 if row i's run has two or more members (keys sorted).
+// The second, a running count of the rows whose run has two or more members,
+// collects those rows in order (and their number, at the last row).
 template <class K>
-__global__ void active_kernel(const K *key, const uint32_t *val, uint64_t n, uint64_t m, uint32_t *active) {
-    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < m;
-         i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        const bool head = run_starts(key, val, n, kFirst<K>, i);
-        const bool next_head = i + 1 == m || run_starts(key, val, n, kFirst<K>, i + 1);
-        active[i] = (head && next_head) ? 0u : 1u;
+struct RunActive {
+    const K *key;
+    const uint32_t *val;
+    uint64_t n, m;
+    __device__ __forceinline__ uint32_t operator()(uint64_t i) const {
+        return run_starts(key, val, n, kFirst<K>, i) && (i + 1 == m || run_starts(key, val, n, kFirst<K>, i + 1)) ? 0u
+                                                                                                                  : 1u;
     }
-}
-
-// Compaction: rows of active runs, in order.  pos = inclusive scan of the
-// flags; flags are recomputed from the keys (the flag array was scanned in place).
+};
 template <class K>
-__global__ void compact_kernel(const K *key, const uint32_t *val, uint64_t n, const uint32_t *A, const uint32_t *pos,
-                               uint64_t m, uint32_t *A2) {
-    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < m;
-         i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        const bool head = run_starts(key, val, n, kFirst<K>, i);
-        const bool next_head = i + 1 == m || run_starts(key, val, n, kFirst<K>, i + 1);
-        if (!(head && next_head)) A2[pos[i] - 1] = A ? A[i] : static_cast<uint32_t>(i);
+struct CollectActive {
+    RunActive<K> active;
+    const uint32_t *A;
+    uint32_t *next, *left;
+    __device__ __forceinline__ void operator()(uint64_t i, uint32_t count) const {
+        if (active(i)) next[count - 1] = A ? A[i] : static_cast<uint32_t>(i);
+        if (i + 1 == active.m) *left = count;
     }
-}
+};
 
 // Keys of a doubling round: (rank of the suffix, rank of the suffix h later).
 __global__ void round_key_kernel(const uint32_t *A, uint64_t m, const uint32_t *sa, const uint32_t *rank,
@@ -392,22 +397,19 @@ unsigned grid_for(uint64_t n, int threads) {
     return static_cast<unsigned>(g < 65536ull * 16 ? (g ? g : 1) : 65536ull * 16);
 }
 
-// Device memory of one build, freed on destruction.
+// Device memory of one build: one allocation (a build of 100 Mbp made 17, of 4.7
+// GB), laid out by taking its pieces twice, the first time to add up their sizes.
 struct DevMem {
-    std::vector<void *> ptrs;
-    cudaError_t err = cudaSuccess;
+    char *base = nullptr;
+    uint64_t used = 0;
     template <class T>
-    T *alloc(uint64_t count) {
-        void *p = nullptr;
-        if (err == cudaSuccess) {
-            err = cudaMalloc(&p, (count ? count : 1) * sizeof(T));
-            if (err == cudaSuccess) ptrs.push_back(p);
-            else p = nullptr;
-        }
-        return static_cast<T *>(p);
+    T *take(uint64_t count) {
+        T *at = reinterpret_cast<T *>(base + used);
+        used += (count * sizeof(T) + 255) & ~255ull;
+        return at;
     }
     ~DevMem() {
-        for (void *p : ptrs) cudaFree(p);
+        if (base) cudaFree(base);
     }
 };
 
@@ -415,32 +417,27 @@ struct DevMem {
 
 // After a sort of the m active rows by key: their suffixes' places and ranks, and
 // the rows of the runs that are left (*left of them) in Anext.
-template <class K>
+template <class K, class F>
 static cudaError_t place_round(const SortBufs &B, int c, const uint32_t *val, uint64_t n, uint64_t m,
                                const uint32_t *Acur, uint32_t *Anext, uint32_t *sa, uint32_t *rank, uint32_t *tmp,
-                               uint32_t *left, cudaStream_t st) {
-    const int T = 256;
+                               uint32_t *left, cudaStream_t st, F &&meanwhile) {
     const K *key = reinterpret_cast<const K *>(B.k[c]);
-    // ranks: the row of the first member of each run of equal keys
-    run_head_kernel<K><<<grid_for(m, T), T, 0, st>>>(key, val, n, m, tmp);
-    device_scan(tmp, tmp, m, true, B.scan_tmp, st, OpMax());
-    place_rank_kernel<<<grid_for(m, T), T, 0, st>>>(Acur, B.v[c], tmp, m, sa, rank);
-    // rows of runs with two or more members stay active
-    active_kernel<K><<<grid_for(m, T), T, 0, st>>>(key, val, n, m, tmp);
-    device_scan(tmp, tmp, m, true, B.scan_tmp, st, OpAdd());
-    compact_kernel<K><<<grid_for(m, T), T, 0, st>>>(key, val, n, Acur, tmp, m, Anext);
-    const cudaError_t e = cudaMemcpyAsync(left, tmp + (m - 1), 4, cudaMemcpyDeviceToHost, st);
+    device_scan_with(RunHead<K>{key, val, n}, PlaceRank{Acur, B.v[c], sa, rank}, m, true, B.scan_tmp, st, OpMax());
+    const RunActive<K> active{key, val, n, m};
+    device_scan_with(active, CollectActive<K>{active, Acur, Anext, tmp}, m, true, B.scan_tmp, st, OpAdd());
+    meanwhile();
+    const cudaError_t e = cudaMemcpyAsync(left, tmp, 4, cudaMemcpyDeviceToHost, st);
     return e != cudaSuccess ? e : cudaStreamSynchronize(st);
 }
 
 // Round 0: every suffix by its first kFirst<K> symbols.
-template <class K>
+template <class K, class F>
 static cudaError_t first_round(const uint8_t *y, uint64_t n, uint32_t *sa, uint32_t *rank, uint32_t *A, uint32_t *tmp,
-                               SortBufs &B, uint32_t *left, cudaStream_t st) {
+                               SortBufs &B, uint32_t *left, cudaStream_t st, F &&meanwhile) {
     const uint64_t N = n + 1;
     first_key_kernel<K><<<grid_for(N, 256), 256, 0, st>>>(y, n, reinterpret_cast<K *>(B.k[0]), B.v[0]);
     const int c = radix_sort<K>(B, N, 2 * kFirst<K>, st);
-    return place_round<K>(B, c, B.v[c], n, N, nullptr, A, sa, rank, tmp, left, st);
+    return place_round<K>(B, c, B.v[c], n, N, nullptr, A, sa, rank, tmp, left, st, meanwhile);
 }
 
 // Texts from which round 0 takes the longer keys: 4^16 strings leave about half
@@ -448,14 +445,16 @@ static cudaError_t first_round(const uint8_t *y, uint64_t n, uint32_t *sa, uint3
 constexpr uint64_t kLongKeys = 1ull << 29;
 
 // Suffix array of y$ (y on the device, codes 0..3, length n) into sa (n + 1 rows).
-// rank, A, A2, tmp: n + 1 words each.
+// rank, A, A2, tmp: n + 1 words each.  meanwhile() runs on the host while the GPU
+// is at round 0.
+template <class F>
 static cudaError_t gpu_suffix_array(const uint8_t *y, uint64_t n, uint32_t *sa, uint32_t *rank, uint32_t *A,
-                                    uint32_t *A2, uint32_t *tmp, SortBufs &B, cudaStream_t st) {
+                                    uint32_t *A2, uint32_t *tmp, SortBufs &B, cudaStream_t st, F &&meanwhile) {
     const uint64_t N = n + 1;
     const bool wide = n >= kLongKeys;
     uint32_t left = 0;
-    cudaError_t e = wide ? first_round<uint64_t>(y, n, sa, rank, A, tmp, B, &left, st)
-                         : first_round<uint32_t>(y, n, sa, rank, A, tmp, B, &left, st);
+    cudaError_t e = wide ? first_round<uint64_t>(y, n, sa, rank, A, tmp, B, &left, st, meanwhile)
+                         : first_round<uint32_t>(y, n, sa, rank, A, tmp, B, &left, st, meanwhile);
     uint32_t b = 1;
     while (b < 32 && (1ull << b) < N) b++;
     uint64_t h = wide ? kFirst<uint64_t> : kFirst<uint32_t>;
@@ -465,7 +464,7 @@ static cudaError_t gpu_suffix_array(const uint8_t *y, uint64_t n, uint32_t *sa, 
         const uint64_t m = left;
         round_key_kernel<<<grid_for(m, 256), 256, 0, st>>>(Acur, m, sa, rank, h, n, b, B.k[0], B.v[0]);
         const int c = radix_sort<uint64_t>(B, m, 2 * b, st);
-        e = place_round<uint64_t>(B, c, nullptr, n, m, Acur, Anext, sa, rank, tmp, &left, st);
+        e = place_round<uint64_t>(B, c, nullptr, n, m, Acur, Anext, sa, rank, tmp, &left, st, [] {});
         uint32_t *t = Acur;
         Acur = Anext;
         Anext = t;
@@ -507,29 +506,40 @@ extern "C" int fm_index_build_gpu(const uint8_t *text, uint64_t n, const fm_buil
     fm_index *ix = nullptr;
     {
         DevMem M;
-        uint8_t *x = M.alloc<uint8_t>(n), *xr = M.alloc<uint8_t>(n);
         const uint64_t W = N > 4 * nb ? N : 4 * nb;  // A, A2, tmp also hold 4 count columns of nb blocks
-        uint32_t *sa = M.alloc<uint32_t>(N), *rank = M.alloc<uint32_t>(N), *A = M.alloc<uint32_t>(W);
-        uint32_t *A2 = M.alloc<uint32_t>(W), *tmp = M.alloc<uint32_t>(W);
-        SortBufs B;
-        B.k[0] = M.alloc<uint64_t>(N);
-        B.k[1] = M.alloc<uint64_t>(N);
-        B.v[0] = M.alloc<uint32_t>(N);
-        B.v[1] = M.alloc<uint32_t>(N);
-        B.counts = M.alloc<uint32_t>(kRsBins * tiles);
         const uint64_t scan_n = kRsBins * tiles > N ? kRsBins * tiles : N;
-        B.scan_tmp = M.alloc<uint32_t>(scan_temp_words(scan_n));
-        uint32_t *blocks = M.alloc<uint32_t>(nb * 16), *samp = M.alloc<uint32_t>(ns);
-        uint32_t *kmer = M.alloc<uint32_t>(kwords);
-        unsigned long long *misc = M.alloc<unsigned long long>(8);
-        cudaError_t e = M.err;
-        if (e == cudaSuccess) {  // N replacement and the reversed text (the input copy is freed at once)
-            uint8_t *d_text = nullptr;
-            e = cudaMalloc(&d_text, n);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(d_text, text, n, cudaMemcpyHostToDevice, st);
+        uint8_t *x, *xr;
+        uint32_t *sa, *rank, *A, *A2, *tmp, *blocks, *samp, *kmer;
+        unsigned long long *misc;
+        SortBufs B;
+        auto lay_out = [&] {
+            M.used = 0;
+            x = M.take<uint8_t>(n);
+            xr = M.take<uint8_t>(n);
+            sa = M.take<uint32_t>(N);
+            rank = M.take<uint32_t>(N);
+            A = M.take<uint32_t>(W);
+            A2 = M.take<uint32_t>(W);
+            tmp = M.take<uint32_t>(W);
+            for (int i = 0; i < 2; i++) {
+                B.k[i] = M.take<uint64_t>(N);
+                B.v[i] = M.take<uint32_t>(N);
+            }
+            B.counts = M.take<uint32_t>(kRsBins * tiles);
+            B.scan_tmp = M.take<uint32_t>(scan_temp_words(scan_n));
+            blocks = M.take<uint32_t>(nb * 16);
+            samp = M.take<uint32_t>(ns);
+            kmer = M.take<uint32_t>(kwords);
+            misc = M.take<unsigned long long>(8);
+        };
+        lay_out();
+        cudaError_t e = cudaMalloc(&M.base, M.used);
+        if (e != cudaSuccess) M.base = nullptr;
+        lay_out();
+        if (e == cudaSuccess) {  // N replacement and the reversed text; the codes as given lie where the sort will write
+            uint8_t *d_text = reinterpret_cast<uint8_t *>(B.k[1]);
+            e = cudaMemcpyAsync(d_text, text, n, cudaMemcpyHostToDevice, st);
             if (e == cudaSuccess) text_kernel<<<grid_for(n, 256), 256, 0, st>>>(d_text, n, o.n_seed, x, xr);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (d_text) cudaFree(d_text);
         }
         if (e == cudaSuccess) e = cudaFuncSetAttribute(rs_scatter_kernel<uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                        static_cast<int>(kRsSmem<uint64_t>));
@@ -545,8 +555,19 @@ extern "C" int fm_index_build_gpu(const uint8_t *text, uint64_t n, const fm_buil
         }
         for (int w = 0; w < 2 && e == cudaSuccess && rc == ALN_OK; w++) {
             const uint8_t *y = w ? xr : x;
-            e = gpu_suffix_array(y, n, sa, rank, A, A2, tmp, B, st);
-            if (e != cudaSuccess) break;
+            e = gpu_suffix_array(y, n, sa, rank, A, A2, tmp, B, st, [&] {
+                if (w) return;
+                try {  // the host image's memory, while the GPU sorts
+                    for (HostText &T : ix->t) {
+                        T.blocks.resize(nb * 16);
+                        T.sa_samp.resize(ns);
+                        T.kmer.resize(kwords);
+                    }
+                } catch (const std::bad_alloc &) {
+                    rc = fail(ALN_ENOMEM, "fm_index_build_gpu: host allocation failed");
+                }
+            });
+            if (e != cudaSuccess || rc != ALN_OK) break;
             // Occ blocks: bit planes and counts, then the counts before each middle row
             cudaMemsetAsync(blocks, 0, nb * 16 * 4, st);
             pack_kernel<<<grid_for(nb * 32, 256), 256, 0, st>>>(y, sa, N, nb, blocks, A, A2);
@@ -581,14 +602,6 @@ extern "C" int fm_index_build_gpu(const uint8_t *text, uint64_t n, const fm_buil
                 next += 4ull * strings;
             }
             if ((e = cudaGetLastError()) != cudaSuccess) break;
-            try {
-                Tt.blocks.resize(nb * 16);
-                Tt.sa_samp.resize(ns);
-                Tt.kmer.resize(kwords);
-            } catch (const std::bad_alloc &) {
-                rc = fail(ALN_ENOMEM, "fm_index_build_gpu: host allocation failed");
-                break;
-            }
             if ((e = cudaMemcpyAsync(Tt.blocks.data(), blocks, nb * 16 * 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess) break;
             if ((e = cudaMemcpyAsync(Tt.sa_samp.data(), samp, ns * 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess) break;
             if (kwords && (e = cudaMemcpyAsync(Tt.kmer.data(), kmer, kwords * 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
