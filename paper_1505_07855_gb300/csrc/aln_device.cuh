@@ -148,6 +148,35 @@ __device__ __forceinline__ void lf1(const DText &T, uint32_t c, uint32_t &lo, ui
     hi = hi4[c];
 }
 
+// occ_before of one base c at offset o of the block, from its half: 3 popcounts
+// (the padding and $ counted as A).
+__device__ __forceinline__ uint32_t occ1_in_half(const HalfBlock &H, uint32_t o, uint32_t c) {
+    const bool up = o >= kHalfRows;
+    const int x = static_cast<int>(up ? o - kHalfRows : o);
+    const uint32_t fl = (c & 1u) ? 0u : 0xFFFFFFFFu, fh = (c & 2u) ? 0u : 0xFFFFFFFFu;
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int g = 0; g < 3; g++) {
+        uint32_t m = __funnelshift_lc(0xFFFFFFFFu, 0u, static_cast<uint32_t>(max(x - 32 * g, 0)));
+        if (!up) m = ~m;
+        cnt += __popc((H.w[g] ^ fl) & (H.w[3 + g] ^ fh) & m);
+    }
+    const uint32_t base = c == 0 ? H.cnt[0] : (c == 1 ? H.cnt[1] : (c == 2 ? H.cnt[2] : H.cnt[3]));
+    return up ? base + cnt : base - cnt;
+}
+
+__device__ __forceinline__ uint32_t c1_of(const DText &T, uint32_t c) {
+    return c == 0 ? T.C1[0] : (c == 1 ? T.C1[1] : (c == 2 ? T.C1[2] : T.C1[3]));
+}
+
+// The lower end of an interval extended by base c: C1[c] + occ_before(c, pos).
+__device__ __forceinline__ uint32_t lf_base(const DText &T, uint32_t c, uint32_t pos) {
+    const uint32_t b = pos / kRowsPerBlock, o = pos - b * kRowsPerBlock;
+    HalfBlock H;
+    load_half(T.blocks, b, o, H);
+    return c1_of(T, c) + occ1_in_half(H, o, c) - (c == 0 && pos > T.primary ? 1u : 0u);
+}
+
 // LF(r) = C1[B[r]] + occ_before(B[r], r) for a row r != primary: the row of the
 // suffix that starts one text position earlier; c = B[r], the base there.
 __device__ __forceinline__ uint32_t lf_row(const DText &T, uint32_t r, uint32_t &c) {
@@ -155,11 +184,7 @@ __device__ __forceinline__ uint32_t lf_row(const DText &T, uint32_t r, uint32_t 
     HalfBlock H;
     load_half(T.blocks, b, o, H);
     c = sym_in_half(H, o);
-    uint32_t occ[4];
-    occ4_in_half(H, o, occ);
-    uint32_t v = occ[c];
-    if (c == 0) v -= (r > T.primary) ? 1u : 0u;
-    return T.C1[c] + v;
+    return c1_of(T, c) + occ1_in_half(H, o, c) - (c == 0 && r > T.primary ? 1u : 0u);
 }
 
 __device__ __forceinline__ uint32_t lf_row(const DText &T, uint32_t r) {

@@ -42,17 +42,50 @@ bool seed_supported(const DIndex &X, const SearchParams &p) {
     return X.lo && min(p.max_gapo, p.z) <= 1u && !p.bounded;
 }
 
-// One thread per read, the tree search; with `seeded`, the block first answers what
-// it can of its reads from seeds, kPlainLanes lanes a read, and its first threads
-// search the rest.  A block then takes a quarter of its threads' number of reads,
-// so that a batch of few reads still has blocks for every SM.
+// One thread per read, the tree search.
+template <int STACK_CAP>
+__device__ __forceinline__ void plain_tree(const DIndex &X, const ReadBatch &rb, const SearchParams &p, uint32_t r,
+                                           uint32_t *sb, uint32_t *sn, aln_read_result *res, aln_hit *hits) {
+    const uint32_t m = rb.len[r];
+    const uint32_t z = rb.z ? rb.z[r] : p.z;
+    const ReadView rv{sb, sn};
+    if (m <= ALN_MAX_READ_LEN && m > 0) load_read(rb, rb.offset[r], m, sb, sn);
+    Search<STACK_CAP> S;
+    S.run(X, rv, m, z, p, res + r, hits + static_cast<uint64_t>(r) * p.hit_cap);
+}
+
+template <int STACK_CAP>
+__global__ void __launch_bounds__(kThreads) aln_plain_kernel(DIndex X, ReadBatch rb, uint32_t n_reads, SearchParams p,
+                                                             aln_read_result *res, aln_hit *hits) {
+    __shared__ uint32_t s_bases[kReadWords * kThreads];
+    __shared__ uint32_t s_nmask[kMaskWords * kThreads];
+    const uint32_t r = blockIdx.x * kThreads + threadIdx.x;
+    if (r >= n_reads) return;
+    plain_tree<STACK_CAP>(X, rb, p, r, s_bases + threadIdx.x, s_nmask + threadIdx.x, res, hits);
+}
+
+// The same after a seed search: the block answers what it can of its reads,
+// kPlainLanes lanes a read, and its first threads search the rest.  A block takes
+// a quarter of its threads' number of reads, so that a batch of few reads still has
+// blocks for every SM.  The tree search is out of line, or its registers would
+// leave room for three blocks on an SM (100 000 reads of 100 bases on 100 Mbp: 1.47 ms
+// in one kernel with it, 0.47 ms so; the tree search alone takes 52 ms).
 constexpr int kPlainLanes = 16;
-constexpr uint32_t kPlainReads = kThreads / 4;    // reads of a seeded block
+constexpr uint32_t kPlainReads = kThreads / 4;
 constexpr uint32_t kPlainTargets = 32, kPlainPlaces = 2048;
 
 template <int STACK_CAP>
-__global__ void __launch_bounds__(kThreads) aln_plain_kernel(const __grid_constant__ DIndex X, ReadBatch rb, uint32_t n_reads, const __grid_constant__ SearchParams p,
-                                                             aln_read_result *res, aln_hit *hits, bool seeded) {
+__device__ __noinline__ void plain_rest(const DIndex &X, const ReadBatch &rb, const SearchParams &p, uint32_t r,
+                                        uint32_t *sb, uint32_t *sn, aln_read_result *res, aln_hit *hits) {
+    plain_tree<STACK_CAP>(X, rb, p, r, sb, sn, res, hits);
+}
+
+template <int STACK_CAP>
+__global__ void __launch_bounds__(kThreads, 5) aln_plain_seed_kernel(const __grid_constant__ DIndex X,
+                                                                     const __grid_constant__ ReadBatch rb,
+                                                                     uint32_t n_reads,
+                                                                     const __grid_constant__ SearchParams p,
+                                                                     aln_read_result *res, aln_hit *hits) {
     __shared__ union {
         SeedRead<kPlainTargets> read[kThreads / kPlainLanes];
         struct {
@@ -60,31 +93,19 @@ __global__ void __launch_bounds__(kThreads) aln_plain_kernel(const __grid_consta
         } tree;
     } sh;
     __shared__ uint32_t s_rest[kPlainReads], s_count;
-    uint32_t r;
-    if (seeded) {
-        if (threadIdx.x == 0) s_count = 0;
-        __syncthreads();
-        const uint32_t group = threadIdx.x / kPlainLanes, first = blockIdx.x * kPlainReads;
-        for (uint32_t i = group; i < kPlainReads; i += kThreads / kPlainLanes) {  // the same rounds for every group
-            const bool active = first + i < n_reads;
-            const bool done = seed_search<kPlainLanes, kPlainTargets, false>(X, rb, p, sh.read[group], first + i, active,
-                                                                             kPlainPlaces, res, hits);
-            if (active && !done && threadIdx.x % kPlainLanes == 0) s_rest[atomicAdd(&s_count, 1u)] = first + i;
-        }
-        __syncthreads();
-        if (threadIdx.x >= s_count) return;
-        r = s_rest[threadIdx.x];
-    } else {
-        r = blockIdx.x * kThreads + threadIdx.x;
-        if (r >= n_reads) return;
+    if (threadIdx.x == 0) s_count = 0;
+    __syncthreads();
+    const uint32_t group = threadIdx.x / kPlainLanes, first = blockIdx.x * kPlainReads;
+    for (uint32_t i = group; i < kPlainReads; i += kThreads / kPlainLanes) {  // the same rounds for every group
+        const bool active = first + i < n_reads;
+        const bool done = seed_search<kPlainLanes, kPlainTargets, false, true>(X, rb, p, sh.read[group], first + i, active,
+                                                                         kPlainPlaces, res, hits);
+        if (active && !done && threadIdx.x % kPlainLanes == 0) s_rest[atomicAdd(&s_count, 1u)] = first + i;
     }
-    const uint32_t m = rb.len[r];
-    const uint32_t z = rb.z ? rb.z[r] : p.z;
-    ReadView rv{sh.tree.bases + threadIdx.x, sh.tree.nmask + threadIdx.x};
-    if (m <= ALN_MAX_READ_LEN && m > 0)
-        load_read(rb, rb.offset[r], m, sh.tree.bases + threadIdx.x, sh.tree.nmask + threadIdx.x);
-    Search<STACK_CAP> S;
-    S.run(X, rv, m, z, p, res + r, hits + static_cast<uint64_t>(r) * p.hit_cap);
+    __syncthreads();
+    if (threadIdx.x < s_count)
+        plain_rest<STACK_CAP>(X, rb, p, s_rest[threadIdx.x], sh.tree.bases + threadIdx.x, sh.tree.nmask + threadIdx.x,
+                              res, hits);
 }
 
 #ifndef ALN_PERSISTENT_MIN_BLOCKS
@@ -879,9 +900,9 @@ constexpr uint32_t kSeedTargets = 32;
 constexpr uint32_t kSeedPlaces = ALN_SEED_PLACES;
 constexpr uint32_t kWidePlaces = 16384;
 
-// Resident blocks per SM: 4 / 5 / 6 take 4.2 / 3.97 / 3.89 ms for 1 M reads of 100
-// bases on 100 Mbp (latency; 6 spills 30 bytes in the gapped path), the wide kernel
-// gains nothing past 5.
+// Resident blocks per SM: 4 / 5 / 6 take 3.36 / 3.08 / 2.98 ms for 1 M reads of 100
+// bases on 100 Mbp and 6.28 / 5.87 / 5.76 ms for 300 000 mates on 3.1 Gbp (latency; 6
+// spills in the gapped path); the wide kernel is the same with 4 and 5.
 #ifndef ALN_SEED_MIN_BLOCKS
 #define ALN_SEED_MIN_BLOCKS 6
 #endif
@@ -1027,9 +1048,10 @@ static cudaError_t launch_cap(const DIndex &X, const ReadBatch &rb, uint32_t n, 
                               aln_read_result *res, aln_hit *hits, uint32_t mode, uint32_t *queue,
                               void *scratch, cudaStream_t st) {
     if (mode == ALN_MODE_PLAIN) {
-        const bool seeded = seed_supported(X, p);
-        const uint32_t each = seeded ? kPlainReads : kThreads;
-        aln_plain_kernel<CAP><<<(n + each - 1) / each, kThreads, 0, st>>>(X, rb, n, p, res, hits, seeded);
+        if (seed_supported(X, p))
+            aln_plain_seed_kernel<CAP><<<(n + kPlainReads - 1) / kPlainReads, kThreads, 0, st>>>(X, rb, n, p, res, hits);
+        else
+            aln_plain_kernel<CAP><<<(n + kThreads - 1) / kThreads, kThreads, 0, st>>>(X, rb, n, p, res, hits);
     } else {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);

@@ -27,8 +27,8 @@
 // Where the tree search of a read of 100 bases expands about 1900 nodes, one after
 // the other, this takes 2 (z + 1) look-ups at once and looks at about ten places
 // (100 Mbp), each a read of the suffix array and of the text.  1 M reads of 100
-// bases at z = 4 on 100 Mbp: 64.9 -> 3.9 ms; 400 000 reads of 36 to 250 bases on
-// 3.1 Gbp: 736 -> 20 ms (profiles/aln_seed.md).  It is bound by the latency of
+// bases at z = 4 on 100 Mbp: 65 -> 3.0 ms; 400 000 reads of 36 to 250 bases on
+// 3.1 Gbp: 725 -> 14-16 ms (profiles/aln_seed.md).  It is bound by the latency of
 // those four dependent random reads and by instruction issue, not by bandwidth.
 #pragma once
 
@@ -52,26 +52,6 @@ constexpr uint32_t kWideRows = 1u << 20;  // a part's rows saturate here
 // and 8 are within 2 % of each other on the 3.1 Gbp batches (1 costs unique reads
 // of 100 Mbp 12 %).
 constexpr uint32_t kManyPlaces = ALN_MANY_PLACES;
-
-// Symbols c in B[0 .. pos-1] of one base.
-__device__ __forceinline__ uint32_t occ1(const DText &T, uint32_t c, uint32_t pos) {
-    const uint32_t b = pos / kRowsPerBlock, o = pos - b * kRowsPerBlock;
-    HalfBlock H;
-    load_half(T.blocks, b, o, H);
-    const bool up = o >= kHalfRows;
-    const int x = static_cast<int>(up ? o - kHalfRows : o);
-    const uint32_t fl = (c & 1u) ? 0u : 0xFFFFFFFFu, fh = (c & 2u) ? 0u : 0xFFFFFFFFu;
-    uint32_t cnt = 0;
-#pragma unroll
-    for (int g = 0; g < 3; g++) {
-        uint32_t m = __funnelshift_lc(0xFFFFFFFFu, 0u, static_cast<uint32_t>(max(x - 32 * g, 0)));
-        if (!up) m = ~m;
-        cnt += __popc((H.w[g] ^ fl) & (H.w[3 + g] ^ fh) & m);
-    }
-    const uint32_t base = c == 0 ? H.cnt[0] : (c == 1 ? H.cnt[1] : (c == 2 ? H.cnt[2] : H.cnt[3]));
-    const uint32_t v = up ? base + cnt : base - cnt;
-    return c == 0 && pos > T.primary ? v - 1u : v;
-}
 
 // Row of the suffix of text w that starts at position pos (0 .. n).
 __device__ __forceinline__ uint32_t row_of(const DIndex &X, int w, uint32_t pos) {
@@ -244,16 +224,21 @@ __device__ __forceinline__ bool gap_fits(const uint2 *text, const Pattern &P, lo
     const uint32_t lo = __funnelshift_r(P.lo[w], P.lo[v], s), hi = __funnelshift_r(P.hi[w], P.hi[v], s);
     const uint32_t nn = __funnelshift_r(P.nn[w], P.nn[v], s);
     const int bound = ahead ? nth_high(mis, F - 1) + 1 : nth_low(mis, F - 1, m);
+    // the 64 bases from 8 before the far word on diagonal d
+    const long long x = d + i - 8;
+    const uint2 *at = text + (x >> 5);
+    const uint32_t t = static_cast<uint32_t>(x & 31);
+    const uint2 a = __ldg(at), b = __ldg(at + 1), c = __ldg(at + 2);
+    const uint32_t lo0 = __funnelshift_r(a.x, b.x, t), lo1 = __funnelshift_r(b.x, c.x, t);
+    const uint32_t hi0 = __funnelshift_r(a.y, b.y, t), hi1 = __funnelshift_r(b.y, c.y, t);
     for (int q = 0; q < 2 * gmost; q++) {
         const int g = (q >> 1) + 1;
         const bool del = q & 1;
         const int window = del ? max(e, 1) : e, gi = del ? 0 : g;
         const uint32_t zone = ahead ? low_mask(max(bound - gi, window))
                                     : low_mask(m - i) & ~low_mask(min(bound, m - window - gi) + gi - i);
-        const long long x = d + i + (del != ahead ? g : -g);
-        const uint2 a = __ldg(text + (x >> 5)), b = __ldg(text + (x >> 5) + 1);
-        const uint32_t t = static_cast<uint32_t>(x & 31);
-        const uint32_t far = (__funnelshift_r(a.x, b.x, t) ^ lo) | (__funnelshift_r(a.y, b.y, t) ^ hi) | nn;
+        const uint32_t by = static_cast<uint32_t>(del != ahead ? 8 + g : 8 - g);
+        const uint32_t far = (__funnelshift_r(lo0, lo1, by) ^ lo) | (__funnelshift_r(hi0, hi1, by) ^ hi) | nn;
         if (__popc(far & zone) + g <= F) return true;
     }
     return false;
@@ -266,7 +251,7 @@ struct SeedRead {
     uint32_t bases[18];              // the read, 2 bits a base (two words past it)
     uint32_t count;                  // targets found (may pass E)
     uint32_t start[E], key[E];       // target start in X; the tree search's candidate key
-    uint32_t row[E], end[E];         // its rows [row, end); end 0: dropped, or another target stands for them
+    uint32_t row[E], end[E];         // its rows [row, end)
 };
 
 // `width` low-order bases from index i of the packed read.
@@ -325,15 +310,15 @@ __device__ __forceinline__ uint32_t key_score(const SearchParams &p, uint32_t ke
     return p.sc_mm * ((key >> 16) & 15u) + p.sc_go * ((key >> 24) & 15u) + p.sc_ge * ((key >> 20) & 15u);
 }
 
+__device__ __forceinline__ uint32_t target_key(uint32_t strand, uint32_t len, uint32_t mm, uint32_t g) {
+    return (strand << 31) | ((mm + g) << 28) | ((g ? 1u : 0u) << 24) | ((g ? g - 1u : 0u) << 20) | (mm << 16) | len;
+}
+
 // A target found: recorded unless it is among the first `have`, those of the
 // rounds before (two lanes may record it in one round; the reduction drops the
 // second).
 template <int E>
-__device__ __forceinline__ void add_target(SeedRead<E> &S, uint32_t have, uint32_t strand, long long a, uint32_t len,
-                                           uint32_t mm, uint32_t g) {
-    const uint32_t key = (strand << 31) | ((mm + g) << 28) | ((g ? 1u : 0u) << 24) | ((g ? g - 1u : 0u) << 20) |
-                         (mm << 16) | len;
-    const uint32_t at = static_cast<uint32_t>(a);
+__device__ __forceinline__ void add_target(SeedRead<E> &S, uint32_t have, uint32_t at, uint32_t key) {
     for (uint32_t j = 0; j < have; j++)
         if (S.start[j] == at && S.key[j] == key) return;
     const uint32_t j = atomicAdd(&S.count, 1u);
@@ -368,11 +353,240 @@ __device__ __forceinline__ void empty_result(aln_read_result *to, uint32_t flags
     *to = out;
 }
 
+// Gapped targets of diagonal d by the lanes of its group, one (gap, side) a lane;
+// returns the fewest differences this lane found.
+template <int G, int E>
+__device__ __forceinline__ uint32_t gap_targets(const uint2 *text, uint32_t n, SeedRead<E> &S, uint32_t have, int m,
+                                             long long d, int first_end, int last_start, uint32_t F, uint32_t gmost,
+                                             int e, SeedZone Z) {
+    const uint32_t strand = Z.reverse ? 1u : 0u;
+    const Pattern &P = S.pat[strand];
+    uint32_t found = 255;
+    for (uint32_t q = threadIdx.x & (G - 1); q < 4 * gmost; q += G) {
+        const int g = static_cast<int>(q >> 2) + 1;
+        const bool del = q & 1u, side = q & 2u;  // side 0: a part lies before the gap, 1: after it
+        const long long other = side == del ? d - g : d + g;
+        const long long a = side ? other : d;
+        const int L = del ? m + g : m - g;
+        int plo = del ? max(e, 1) : e;
+        int phi = del ? m - plo : m - plo - g;
+        if (side) phi = min(phi, last_start - (del ? 0 : g));
+        else plo = max(plo, first_end);
+        if (static_cast<uint32_t>(g) > F || L < 1 || a < 0 || a + L > static_cast<long long>(n) || plo > phi) continue;
+        uint32_t pre[kPlaneWords], suf[kPlaneWords];  // mismatches on the prefix's and on the suffix's diagonal
+        mismatches(text, P, a, m, pre);
+        mismatches(text, P, side ? d : other, m, suf);
+        const uint32_t f = best_gap(pre, suf, m, g, del, plo, phi, F - g, Z);
+        if (f != 0xFFFFFFFFu) {
+            add_target(S, have, static_cast<uint32_t>(a),
+                       target_key(strand, static_cast<uint32_t>(L), f, static_cast<uint32_t>(g)));
+            found = min(found, f + static_cast<uint32_t>(g));
+        }
+    }
+    return found;
+}
+
+template <int G, int E>
+__device__ __noinline__ uint32_t gap_targets_call(const uint2 *text, uint32_t n, SeedRead<E> &S, uint32_t have, int m,
+                                                  long long d, int first_end, int last_start, uint32_t F, uint32_t gmost,
+                                                  int e, SeedZone Z) {
+    return gap_targets<G, E>(text, n, S, have, m, d, first_end, last_start, F, gmost, e, Z);
+}
+
+// Bitonic sort of a read's first P entries (a power of two, the same for every
+// group of the warp) by its G lanes; less(i, j) compares two entries.
+template <int G, int E, class Less>
+__device__ __forceinline__ void sort_targets(SeedRead<E> &S, uint32_t P, Less less) {
+    const uint32_t l = threadIdx.x & (G - 1);
+    for (uint32_t k = 2; k <= P; k <<= 1)
+        for (uint32_t j = k >> 1; j; j >>= 1) {
+            for (uint32_t i = l; i < P / 2; i += G) {
+                const uint32_t x = ((i & ~(j - 1u)) << 1) | (i & (j - 1u)), y = x | j;
+                if (less(y, x) == ((x & k) == 0)) {
+                    const uint32_t s = S.start[x], t = S.key[x], r = S.row[x], e = S.end[x];
+                    S.start[x] = S.start[y];
+                    S.key[x] = S.key[y];
+                    S.row[x] = S.row[y];
+                    S.end[x] = S.end[y];
+                    S.start[y] = s;
+                    S.key[y] = t;
+                    S.row[y] = r;
+                    S.end[y] = e;
+                }
+            }
+            __syncwarp();
+        }
+}
+
+// The entries of the first P that keep(e) holds for move to the front, in order;
+// the others become entries that sort last.  Returns how many are kept.
+template <int G, int E, class Keep>
+__device__ __forceinline__ uint32_t pack_targets(SeedRead<E> &S, uint32_t P, unsigned group_lanes, Keep keep) {
+    const uint32_t l = threadIdx.x & (G - 1);
+    const unsigned before = (1u << (threadIdx.x & 31u)) - 1u;
+    uint32_t n = 0;
+    for (uint32_t i = 0; i < P; i += G) {  // an entry moves to a place at or before its own: behind what is still to be read
+        const uint32_t e = i + l;
+        const bool k = e < P && keep(e);
+        uint32_t s = 0, t = 0, r = 0, d = 0;
+        if (k) {
+            s = S.start[e];
+            t = S.key[e];
+            r = S.row[e];
+            d = S.end[e];
+        }
+        __syncwarp();
+        const unsigned kept = __ballot_sync(0xFFFFFFFFu, k) & group_lanes;
+        if (k) {
+            const uint32_t to = n + __popc(kept & before);
+            S.start[to] = s;
+            S.key[to] = t;
+            S.row[to] = r;
+            S.end[to] = d;
+        }
+        n += __popc(kept);
+        __syncwarp();
+    }
+    for (uint32_t e = l; e < P; e += G)
+        if (e >= n) {
+            S.start[e] = S.end[e] = 0;
+            S.key[e] = S.row[e] = 0xFFFFFFFFu;
+        }
+    __syncwarp();
+    return n;
+}
+
+// The result of a read from its cnt recorded targets with at most F differences:
+// intervals, merged hits, strata, order.  Warp-wide, a group each; true if
+// written (write, and no more hits than the tree search keeps).  By sorting: a
+// read in a repeat has hundreds of targets, and comparing each with each kept one
+// warp busy for milliseconds after the others had gone.
+template <int G, int E, bool SCORE>
+__device__ __noinline__ bool reduce_targets(const DIndex &X, const SearchParams &p, SeedRead<E> &S, uint32_t r,
+                                            uint32_t cnt, uint32_t F, bool write, unsigned group_lanes,
+                                            aln_read_result *res, aln_hit *hits) {
+    constexpr uint32_t kNone = 0xFFFFFFFFu, kTarget = 0x8000FFFFu;  // a key's strand and length
+    const uint32_t l = threadIdx.x & (G - 1), n = X.t[0].n;
+    const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, cnt);
+    uint32_t P = 2;
+    while (P < most) P <<= 1;
+    // targets above the final budget leave; rows of the others
+    for (uint32_t e = l; e < P; e += G) {
+        uint32_t key = kNone, row = kNone;
+        if (e < cnt && key_diffs(S.key[e]) <= F) {
+            key = S.key[e];
+            const uint32_t a = S.start[e];
+            row = (key >> 31) ? row_of(X, 0, a) : row_of(X, 1, n - a - (key & 0xFFFFu));
+        }
+        S.key[e] = key;
+        S.row[e] = row;
+        S.end[e] = 0;
+    }
+    __syncwarp();
+    // each target once, with its least witness (a part may have seen another place
+    // for the gap than the best one)
+    sort_targets<G, E>(S, P, [&](uint32_t i, uint32_t j) {
+        const uint32_t a = S.key[i] & kTarget, b = S.key[j] & kTarget;
+        if (a != b) return a < b;
+        return S.row[i] != S.row[j] ? S.row[i] < S.row[j] : S.key[i] < S.key[j];
+    });
+    uint32_t have = pack_targets<G, E>(S, P, group_lanes, [&](uint32_t e) {
+        return S.row[e] != kNone &&
+               (e == 0 || S.row[e - 1] != S.row[e] || ((S.key[e - 1] ^ S.key[e]) & kTarget) != 0);
+    });
+    // equal targets of several places lie in neighbouring rows: the first of a run
+    // stands for it
+    for (uint32_t e = l; e < have; e += G) {
+        const uint32_t key = S.key[e];
+        const bool joins = e > 0 && S.row[e - 1] + 1u == S.row[e] && S.key[e - 1] == key &&
+                           same_text(X.text, S.start[e - 1], S.start[e], key & 0xFFFFu);
+        S.end[e] = joins ? 1u : 0u;
+    }
+    __syncwarp();
+    for (uint32_t e = l; e < have; e += G)
+        if (!S.end[e]) {
+            uint32_t end = S.row[e] + 1u;
+            for (uint32_t j = e + 1; j < have && S.end[j]; j++) end++;
+            S.start[e] = end;  // the target's start is not needed any more
+        }
+    __syncwarp();
+    for (uint32_t e = l; e < have; e += G) S.end[e] = S.end[e] ? 0u : S.start[e];
+    __syncwarp();
+    have = pack_targets<G, E>(S, P, group_lanes, [&](uint32_t e) { return S.end[e] != 0u; });
+    // hits of equal rows on a strand (targets of several lengths) keep the least (score, witness)
+    sort_targets<G, E>(S, P, [&](uint32_t i, uint32_t j) {
+        const uint32_t a = S.key[i] >> 31, b = S.key[j] >> 31;
+        if (a != b) return a < b;
+        if (S.row[i] != S.row[j]) return S.row[i] < S.row[j];
+        if (S.end[i] != S.end[j]) return S.end[i] < S.end[j];
+        if (SCORE && key_score(p, S.key[i]) != key_score(p, S.key[j])) return key_score(p, S.key[i]) < key_score(p, S.key[j]);
+        return S.key[i] < S.key[j];
+    });
+    have = pack_targets<G, E>(S, P, group_lanes, [&](uint32_t e) {
+        return S.row[e] != kNone && (e == 0 || S.row[e - 1] != S.row[e] || S.end[e - 1] != S.end[e] ||
+                                     ((S.key[e - 1] ^ S.key[e]) >> 31) != 0);
+    });
+    write = write && have <= static_cast<uint32_t>(kCandCap);  // more than that the tree search flags
+    // the order (diffs or score, strand, k, l)
+    auto value = [&](uint32_t e) { return SCORE ? key_score(p, S.key[e]) : key_diffs(S.key[e]); };
+    sort_targets<G, E>(S, P, [&](uint32_t i, uint32_t j) {
+        const bool in = S.row[i] != kNone, jn = S.row[j] != kNone;
+        if (!in || !jn) return in && !jn;
+        const uint32_t a = (value(i) << 1) | (S.key[i] >> 31), b = (value(j) << 1) | (S.key[j] >> 31);
+        if (a != b) return a < b;
+        return S.row[i] != S.row[j] ? S.row[i] < S.row[j] : S.end[i] < S.end[j];
+    });
+    uint32_t s1 = have ? value(0) : kNone, s2 = kNone, best = 255, c0 = 0, c1 = 0, n1 = 0, n2 = 0;
+    if (SCORE) {
+        for (uint32_t e = l; e < have; e += G)
+            if (value(e) > s1) s2 = min(s2, value(e));
+        s2 = group_min<G>(s2);
+    } else {
+        s2 = s1 + 1u;
+    }
+    for (uint32_t e = l; e < have; e += G) {
+        const uint32_t v = value(e), w = S.end[e] - S.row[e];
+        if (v == s1) {
+            c0 += w;
+            n1++;
+            best = min(best, key_diffs(S.key[e]));
+        } else if (v == s2) {
+            c1 += w;
+            n2++;
+        }
+    }
+    best = group_min<G>(best);
+    c0 = group_sum<G>(c0);
+    c1 = group_sum<G>(c1);
+    n1 = group_sum<G>(n1);
+    n2 = group_sum<G>(n2);
+    const bool many = SCORE && p.max_best && c0 > p.max_best;
+    const uint32_t listed = SCORE ? n1 + (many ? 0u : n2) : have;
+    if (write)
+        for (uint32_t e = l; e < min(listed, p.hit_cap); e += G)
+            put_hit(hits + static_cast<uint64_t>(r) * p.hit_cap + e, S.row[e], S.end[e] - 1u, S.key[e]);
+    if (write && l == 0) {
+        aln_read_result out;
+        const bool any = listed > 0;
+        const uint32_t flags = (many ? ALN_FLAG_MANY_BEST : 0u) | (listed > p.hit_cap ? ALN_FLAG_HIT_OVERFLOW : 0u);
+        out.c0 = any ? c0 : 0u;
+        out.c1 = any ? c1 : 0u;
+        out.n_hits = static_cast<uint8_t>(min(listed, p.hit_cap));
+        out.d_best = static_cast<uint8_t>(any ? best : 255u);
+        out.best_score = static_cast<uint8_t>(SCORE ? (any ? min(s1, 254u) : 255u) : 0u);
+        out.flags = static_cast<uint8_t>(flags);
+        res[r] = out;
+    }
+    return write;
+}
+
 // Search of one read by the G lanes of a group; all 32 lanes of the warp call it
 // together (other groups with their own reads, or with active = false).  True
 // if the read's result was written; false if it has too many places or targets
-// for this form (nothing is written then).
-template <int G, int E, bool SCORE>
+// for this form (nothing is written then).  CALL: the gapped stage out of line
+// (1 M reads take 3.37 ms with it and 2.93 without; in the plain kernel, whose tree
+// search takes its registers, 100 000 take 0.48 ms with it and 1.25 without).
+template <int G, int E, bool SCORE, bool CALL = false>
 __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchParams &p, SeedRead<E> &S, uint32_t r,
                             bool active, uint32_t max_places, aln_read_result *res, aln_hit *hits) {
     constexpr unsigned FULL = 0xFFFFFFFFu;
@@ -507,8 +721,8 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
             if (!__any_sync(FULL, go)) break;
             if (go) {
                 const uint32_t c = ((S.bases[next >> 4] >> (2 * (next & 15u))) & 3u) ^ (strand ? 3u : 0u);
-                lo = X.t[0].C1[c] + occ1(X.t[0], c, lo);
-                hi = X.t[0].C1[c] + occ1(X.t[0], c, hi);
+                lo = lf_base(X.t[0], c, lo);
+                hi = lf_base(X.t[0], c, hi);
                 width = hi > lo ? min(hi - lo, kWideRows) : 0u;
                 next += strand ? 1u : ~0u;
                 off--;
@@ -560,16 +774,10 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
                 mismatches(X.text, P, d, m, mis);
                 live = count_in(mis, qs, qe) == 0;  // else another part leads to what this diagonal has
             }
-            // of the lanes on one diagonal the first looks on, for all their parts
-            const unsigned long long tag = live ? (static_cast<unsigned long long>(d + 16) << 8) |
-                                                      ((threadIdx.x & 31u) / G * 2 + cs)
-                                                : ~0ull - (threadIdx.x & 31u);
-            const unsigned same = __match_any_sync(FULL, tag);
-            const int first_end = static_cast<int>(__reduce_min_sync(same, static_cast<unsigned>(qe)));
-            const int last_start = static_cast<int>(__reduce_max_sync(same, static_cast<unsigned>(qs)));
-            live = live && static_cast<uint32_t>(__ffs(same) - 1) == (threadIdx.x & 31u);
             if (live && d >= 0 && d + m <= static_cast<long long>(n)) {
-                mm = count_in(mis, 0, m);
+                mm = 0;
+#pragma unroll
+                for (int w = 0; w < kPlaneWords; w++) mm += __popc(mis[w]);
                 if (p.seed_len && mm <= z) {
                     const SeedZone Z = zone(cs);
                     if (count_in(mis, Z.from, Z.to) > Z.most) mm = 255;
@@ -577,57 +785,45 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
             }
             dmin = min(dmin, group_min<G>(mm));
             if (!exhaustive) F = min(z, dmin + 1);
-            if (live && mm <= F) add_target(S, have, cs, d, static_cast<uint32_t>(m), mm, 0u);
-            // gapped targets: a diagonal whose prefix or suffix leaves differences for a
-            // gap is looked at by the whole group, one (gap, side) a lane
+            // gapless targets, one diagonal after the other (several parts lead to a
+            // read's own place in one round): the group looks whether it has it already
+            for (unsigned left = __ballot_sync(FULL, live && mm <= F) & group_lanes; __any_sync(FULL, left != 0);) {
+                const int src = left ? __ffs(left) - 1 : static_cast<int>(threadIdx.x & 31u);
+                const long long dd = __shfl_sync(FULL, d, src);
+                const uint32_t ds = __shfl_sync(FULL, cs, src), dm = __shfl_sync(FULL, mm, src);
+                const bool same = dd == d && ds == cs;
+                const uint32_t key = target_key(ds, static_cast<uint32_t>(m), dm, 0u);
+                bool known = false;
+                for (uint32_t j = l; left && j < have; j += G)
+                    known = known || (S.start[j] == static_cast<uint32_t>(dd) && S.key[j] == key);
+                known = (__ballot_sync(FULL, known) & group_lanes) != 0;
+                if (left && !known && src == static_cast<int>(threadIdx.x & 31u))
+                    add_target(S, 0u, static_cast<uint32_t>(dd), key);
+                left &= ~__ballot_sync(FULL, same);
+            }
+            // gapped targets: a diagonal that a gap may lead to or from is looked at by
+            // the whole group, for the parts that found it in this round
             const uint32_t gmost = p.max_gapo ? min(F, p.max_gape + 1u) : 0u;
             bool want = false;
             if (live && gmost) {
                 const int f = static_cast<int>(F), gm = static_cast<int>(gmost), e = static_cast<int>(p.e);
-                want = (count_in(mis, 0, first_end) < F && gap_fits(X.text, P, d, m, mis, f, gm, e, false)) ||
-                       (count_in(mis, last_start, m) < F && gap_fits(X.text, P, d, m, mis, f, gm, e, true));
+                want = (count_in(mis, 0, qs) < F && gap_fits(X.text, P, d, m, mis, f, gm, e, false)) ||
+                       (count_in(mis, qe, m) < F && gap_fits(X.text, P, d, m, mis, f, gm, e, true));
             }
             uint32_t dgap = 255;
-            for (unsigned left = __ballot_sync(FULL, want) & group_lanes; __any_sync(FULL, left != 0); left &= left - 1) {
+            for (unsigned left = __ballot_sync(FULL, want) & group_lanes; __any_sync(FULL, left != 0);) {
                 const int src = left ? __ffs(left) - 1 : static_cast<int>(threadIdx.x & 31u);
-                uint32_t mo[kPlaneWords], md[kPlaneWords];
-#pragma unroll
-                for (int w = 0; w < kPlaneWords; w++) md[w] = __shfl_sync(FULL, mis[w], src);
                 const long long dd = __shfl_sync(FULL, d, src);
                 const uint32_t ds = __shfl_sync(FULL, cs, src);
-                const int fe = __shfl_sync(FULL, first_end, src), ls = __shfl_sync(FULL, last_start, src);
-                SeedZone Z = zone(ds);
-                for (uint32_t q = l; left && q < 4 * gmost; q += G) {
-                    const int g = static_cast<int>(q >> 2) + 1;
-                    const bool del = q & 1u, side = q & 2u;  // side 0: a part lies before the gap, 1: after it
-                    const uint32_t fixed = side ? count_in(md, ls, m) : count_in(md, 0, fe);
-                    const long long other = side == del ? dd - g : dd + g;
-                    const long long a = side ? other : dd;
-                    const int L = del ? m + g : m - g;
-                    int plo = del ? max(static_cast<int>(p.e), 1) : static_cast<int>(p.e);
-                    int phi = del ? m - plo : m - plo - g;
-                    if (side) phi = min(phi, ls - (del ? 0 : g));
-                    else plo = max(plo, fe);
-                    if (fixed + g > F || L < 1 || a < 0 || a + L > static_cast<long long>(n) || plo > phi) continue;
-                    mismatches(X.text, S.pat[ds], other, m, mo);
-                    if (side) {  // the prefix's mismatches, then the suffix's
-#pragma unroll
-                        for (int w = 0; w < kPlaneWords; w++) {
-                            const uint32_t t = mo[w];
-                            mo[w] = md[w];
-                            md[w] = t;
-                        }
-                    }
-                    const uint32_t f = best_gap(md, mo, m, g, del, plo, phi, F - g, Z);
-                    if (side) {
-#pragma unroll
-                        for (int w = 0; w < kPlaneWords; w++) md[w] = mo[w];
-                    }
-                    if (f != 0xFFFFFFFFu) {
-                        add_target(S, have, ds, a, static_cast<uint32_t>(L), f, static_cast<uint32_t>(g));
-                        dgap = min(dgap, f + static_cast<uint32_t>(g));
-                    }
+                const bool same = want && dd == d && ds == cs;
+                const int fe = static_cast<int>(group_min<G>(same ? static_cast<uint32_t>(qe) : 255u));
+                const int ls = 255 - static_cast<int>(group_min<G>(same ? 255u - static_cast<uint32_t>(qs) : 255u));
+                if (left) {
+                    const int e = static_cast<int>(p.e);
+                    dgap = min(dgap, CALL ? gap_targets_call<G, E>(X.text, n, S, have, m, dd, fe, ls, F, gmost, e, zone(ds))
+                                          : gap_targets<G, E>(X.text, n, S, have, m, dd, fe, ls, F, gmost, e, zone(ds)));
                 }
+                left &= ~__ballot_sync(FULL, same);
             }
             dmin = min(dmin, group_min<G>(dgap));
             if (!exhaustive) F = min(z, dmin + 1);
@@ -670,124 +866,9 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
         }
         return (search && !failed) || answer;
     }
-    // targets above the final budget and second records leave; rows of the others
-    for (uint32_t e = l; e < cnt; e += G) {
-        const uint32_t key = S.key[e], a = S.start[e];
-        bool keep = key_diffs(key) <= F;
-        for (uint32_t j = 0; j < e && keep; j++) keep = !(S.start[j] == a && S.key[j] == key);
-        uint32_t row = 0xFFFFFFFFu;
-        if (keep) row = (key >> 31) ? row_of(X, 0, a) : row_of(X, 1, n - a - (key & 0xFFFFu));
-        S.row[e] = row;
-        S.end[e] = keep ? 1u : 0u;
-    }
-    __syncwarp();
-    // the first row of a run of equal targets stands for the run
-    for (uint32_t e = l; e < cnt; e += G) {
-        if (!S.end[e]) continue;
-        const uint32_t key = S.key[e], row = S.row[e], a = S.start[e];
-        uint32_t top = row;
-        bool first = true;
-        for (uint32_t j = 0; j < cnt && first; j++)
-            first = !(S.row[j] + 1u == row && S.row[j] != 0xFFFFFFFFu && S.key[j] == key &&
-                      same_text(X.text, S.start[j], a, key & 0xFFFFu));
-        bool more = first;
-        while (more) {
-            more = false;
-            for (uint32_t j = 0; j < cnt; j++)
-                if (S.row[j] == top + 1u && S.key[j] == key && S.row[j] != 0xFFFFFFFFu &&
-                    same_text(X.text, S.start[j], a, key & 0xFFFFu)) {
-                    top++;
-                    more = true;
-                    break;
-                }
-        }
-        S.end[e] = first ? top + 1u : 0u;  // no other lane reads it before the barrier
-    }
-    __syncwarp();
-    // hits of equal rows on a strand keep the least (score, witness)
-    uint32_t drop = 0, kept = 0, s1 = 0xFFFFFFFFu;
-    for (uint32_t e = l, i = 0; e < cnt; e += G, i++) {
-        const uint32_t key = S.key[e], row = S.row[e], end = S.end[e];
-        bool keep = end != 0u;
-        for (uint32_t j = 0; j < cnt && keep; j++)
-            if (j != e && S.row[j] == row && S.end[j] == end && (S.key[j] >> 31) == (key >> 31)) {
-                if (SCORE) {
-                    const uint32_t a = key_score(p, S.key[j]), c = key_score(p, key);
-                    keep = !(a < c || (a == c && S.key[j] < key));
-                } else {
-                    keep = !(S.key[j] < key);
-                }
-            }
-        if (!keep) drop |= 1u << i;
-        else if (SCORE) s1 = min(s1, key_score(p, key));
-        if (keep) kept++;
-    }
-    __syncwarp();
-    for (uint32_t e = l, i = 0; e < cnt; e += G, i++)
-        if ((drop >> i) & 1u) S.end[e] = 0u;
-    kept = group_sum<G>(kept);
-    if (kept > static_cast<uint32_t>(kCandCap)) failed = true;  // the tree search flags it
-    __syncwarp();
-    uint32_t best = 255, c0 = 0, c1 = 0, s2 = 0xFFFFFFFFu;
-    if (SCORE) {
-        s1 = group_min<G>(s1);
-        for (uint32_t e = l; e < cnt; e += G)
-            if (S.end[e]) {
-                const uint32_t sc = key_score(p, S.key[e]);
-                if (sc > s1) s2 = min(s2, sc);
-                else best = min(best, key_diffs(S.key[e]));
-            }
-        s2 = group_min<G>(s2);
-    } else {
-        for (uint32_t e = l; e < cnt; e += G)
-            if (S.end[e]) best = min(best, key_diffs(S.key[e]));
-    }
-    best = group_min<G>(best);
-    for (uint32_t e = l; e < cnt; e += G)
-        if (S.end[e]) {
-            const uint32_t w = S.end[e] - S.row[e];
-            const uint32_t v = SCORE ? key_score(p, S.key[e]) : key_diffs(S.key[e]);
-            if (v == (SCORE ? s1 : best)) c0 += w;
-            else if (v == (SCORE ? s2 : best + 1)) c1 += w;
-        }
-    c0 = group_sum<G>(c0);
-    c1 = group_sum<G>(c1);
-    const bool many = SCORE && p.max_best && c0 > p.max_best;
-    uint32_t listed = 0;
-    const bool write = search && !failed;
-    for (uint32_t e = l; e < cnt && write; e += G) {
-        if (!S.end[e]) continue;
-        const uint32_t key = S.key[e], row = S.row[e], end = S.end[e];
-        const uint32_t v = SCORE ? key_score(p, key) : key_diffs(key);
-        if (SCORE && v != s1 && (many || v != s2)) continue;
-        listed++;
-        uint32_t rank = 0;  // hits before it in the order (diffs or score, strand, k, l)
-        for (uint32_t j = 0; j < cnt; j++) {
-            if (!S.end[j] || j == e) continue;
-            const uint32_t kj = S.key[j], vj = SCORE ? key_score(p, kj) : key_diffs(kj);
-            const uint32_t oj = (vj << 1) | (kj >> 31), oe = (v << 1) | (key >> 31);
-            rank += oj < oe || (oj == oe && (S.row[j] < row || (S.row[j] == row && S.end[j] < end))) ? 1u : 0u;
-        }
-        if (rank < p.hit_cap) {
-            put_hit(hits + static_cast<uint64_t>(r) * p.hit_cap + rank, row, end - 1u, key);
-        }
-    }
-    listed = group_sum<G>(listed);
+    const bool written = reduce_targets<G, E, SCORE>(X, p, S, r, cnt, F, search && !failed, group_lanes, res, hits);
     if (answer && l == 0) empty_result<SCORE>(res + r, flags);
-    if (write && l == 0) {
-        aln_read_result out;
-        const bool any = listed > 0;
-        if (many) flags |= ALN_FLAG_MANY_BEST;
-        if (listed > p.hit_cap) flags |= ALN_FLAG_HIT_OVERFLOW;
-        out.c0 = any ? c0 : 0u;
-        out.c1 = any ? c1 : 0u;
-        out.n_hits = static_cast<uint8_t>(min(listed, p.hit_cap));
-        out.d_best = static_cast<uint8_t>(any ? best : 255u);
-        out.best_score = static_cast<uint8_t>(SCORE ? (any ? min(s1, 254u) : 255u) : 0u);
-        out.flags = static_cast<uint8_t>(flags);
-        res[r] = out;
-    }
-    return write || answer;
+    return written || answer;
 }
 
 }  // namespace aln

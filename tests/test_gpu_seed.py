@@ -132,7 +132,8 @@ def test_seed_search_against_the_oracle(torch, strata):
 
 def test_reads_left_to_the_tree_search(torch):
     """A text of one letter but for a random stretch: its reads have too many
-    places for the seed search, in a batch with reads that have few."""
+    places for the seed search, in a batch with reads that have few: of up to
+    2048 reads (the heavy phase in one kernel) and of more."""
     rng = Rng(5, "left")
     text = np.zeros(40_000, np.uint8)
     text[10_000:30_000] = reference_iid(20_000, rng.sub("t"))
@@ -140,11 +141,12 @@ def test_reads_left_to_the_tree_search(torch):
     a = simulate_reads(text[10_000:30_000], 700, (50, 100), rng.sub("a"), z=2)
     b = Reads(np.zeros(64 * 40, np.uint8), np.arange(64, dtype=np.uint64) * np.uint64(40),
               np.full(64, 40, np.uint16), np.full(64, 2, np.uint8), np.zeros(64, np.int64), np.zeros(64, np.uint8))
-    reads = Reads.concat([a, b]).subset(np.random.default_rng(1).permutation(a.n + b.n))
+    once = Reads.concat([a, b]).subset(np.random.default_rng(1).permutation(a.n + b.n))
     p = aln.Params(z=2, hit_cap=16, mode=aln.MODE_PERSISTENT)
-    for heavy in (0, 1, 0xFFFFFFFF):
-        p.heavy_after, p.work_limit = heavy, 0
-        got = al.align(reads.codes, reads.offsets, reads.lens, p)
-        p.work_limit = TREE
-        _same(got, al.align(reads.codes, reads.offsets, reads.lens, p), 16, heavy)
-    assert (got[0]["c0"] > 9000).sum() >= 64
+    for reads in (once, Reads.concat([once] * 4)):
+        for heavy in (0, 1, 0xFFFFFFFF):
+            p.heavy_after, p.work_limit = heavy, 0
+            got = al.align(reads.codes, reads.offsets, reads.lens, p)
+            p.work_limit = TREE
+            _same(got, al.align(reads.codes, reads.offsets, reads.lens, p), 16, heavy)
+        assert (got[0]["c0"] > 9000).sum() >= 64
