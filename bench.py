@@ -37,7 +37,7 @@ BYTES_PER_LOOKUP = 64
 # of each workload (a few hundred thousand reads, scaled per read; the profile
 # summaries under profiles/ give the command).  Used only while the kernel
 # sources hash to the value they had at capture time.
-KERNEL_SOURCES = ("aln_device.cuh", "aln_search.cuh", "aln_flat.cuh", "aln_kernels.cu")
+KERNEL_SOURCES = ("aln_device.cuh", "aln_search.cuh", "aln_seed.cuh", "aln_flat.cuh", "aln_kernels.cu")
 TRAFFIC_CAPTURE = {  # workload -> capture; the profile summaries give the commands
     # 300 000 of the 1 M reads: 6.778 GB read + 0.254 GB written in one launch
     "chr100": {"src_sha256_16": "b5a44875db83a4ce", "dram_bytes_per_read": 23441},
@@ -385,11 +385,28 @@ def accuracy_report(w, outp, pos, npos, hit_cap, valid):
     return out
 
 
+def seed_blocks(reads, n_hits):
+    """Random 64-byte blocks per read that the seed search cannot do without: a
+    k-mer entry for each (strand, error-free part) of the z + 1 parts, and for each
+    hit its suffix-array entry, the text under it and its row's inverse entry."""
+    text = np.ceil((reads.lens.astype(np.float64) / 32 + 1) * 8 / BYTES_PER_LOOKUP).mean()
+    return float(2 * (reads.z.astype(np.float64).mean() + 1) + n_hits.astype(np.float64).mean() * (2 + text))
+
+
+def derived_index_bytes(n):
+    """Bytes of the arrays the upload derives from an index of n bases (aln_derive.cu):
+    both suffix arrays, a quarter of their inverses, the text's planes, the k-mer table."""
+    k = 1
+    while k < 16 and 4 ** (k + 1) <= 4 * (n + 1):
+        k += 1
+    return 8 * n + 2 * n + n // 4 + 4 * 4 ** k
+
+
 def roofline(lookups_per_read, n, ms, probes, index_bytes, workload_name):
-    """Achieved algorithmic bytes/s of the search (64 B per Occ lookup of the
-    oracle's canonical count, the D scans included) against the random 64-byte
-    gather rate of the memory that serves the index: L2 when the searched index
-    (Occ blocks + prefix-trie tables of both texts) fits in L2, else HBM; the
+    """Achieved algorithmic bytes/s of the search (64 B per random block read it
+    cannot do without: seed_blocks) against the random 64-byte gather rate of the
+    memory that serves the index: L2 when the searched index (derived arrays, Occ
+    blocks and prefix-trie tables of both texts) fits in L2, else HBM; the
     fraction of the streaming copy peak is reported beside it."""
     copy_peak, src = _peaks()
     bytes_per_read = lookups_per_read * BYTES_PER_LOOKUP
@@ -409,7 +426,7 @@ def roofline(lookups_per_read, n, ms, probes, index_bytes, workload_name):
                            else f"streaming copy peak ({src})",
             "index_bytes": int(index_bytes), "copy_peak": copy_peak, "copy_peak_source": src,
             "frac_of_copy_peak": achieved / copy_peak, "bytes_per_read": bytes_per_read,
-            "occ_lookups_per_s": lookups_per_read * n / (ms / 1000)}
+            "block_reads_per_s": lookups_per_read * n / (ms / 1000)}
 
 
 def workload_config(name, w, n_per_step, ws, mode="persistent"):
@@ -425,11 +442,13 @@ def workload_config(name, w, n_per_step, ws, mode="persistent"):
 
 
 def search_launches(aln, params, scratch=True):
-    """Kernels one search launches (the same list whether launched directly or
-    replayed from a graph): the plain form one; the persistent form the search,
-    with scratch the D pre-pass and the two visit-order kernels before it, and
-    unless the heavy phase is off its start kernel and one pass and one decide
-    kernel per deepening pass after it."""
+    """Kernels one search of more than 2048 reads launches (the same list whether
+    launched directly or replayed from a graph): the plain form one; the persistent
+    form the tree search, with scratch three before it (the seed search, its wide
+    form and the D scan of the rest; of limits it does not take, the D pre-pass and
+    the two visit-order kernels), and unless the heavy phase is off its start kernel
+    and one pass and one decide kernel per deepening pass after it (one kernel in
+    all for a seed search of at most 2048 reads)."""
     if params.mode == aln.MODE_PLAIN:
         return 1
     n = 1
@@ -552,7 +571,7 @@ def human_phase(args, aln, torch, dev, stream, flush):
     out["index_build"] = {"where": "gpu (fm_index_build_gpu)", "s": time.time() - t0}
     dix = hix.to_device(dev.index)
     info = dix.info()
-    index_bytes = 2 * (info["occ_bytes"] + info["kmer_bytes"])
+    index_bytes = 2 * (info["occ_bytes"] + info["kmer_bytes"]) + derived_index_bytes(info["n"])
     del hix
     al = aln.Aligner(dix)
     hit_cap = 32
@@ -649,7 +668,8 @@ def human_phase(args, aln, torch, dev, stream, flush):
             par["rows_above_2_31"] = int((hq[sel][np.arange(hit_cap)[None, :] < rq[sel]["n_hits"][:, None]]["l"]
                                           >= 2 ** 31).sum())
             b["parity"] = par
-            b["roofline"] = roofline(float(look.mean()), n, ms_p, args._probes, index_bytes, "human_" + name)
+            b["roofline"] = roofline(seed_blocks(w.reads, rq["n_hits"]), n, ms_p, args._probes, index_bytes, "human_" + name)
+            b["roofline"]["tree_occ_lookups_per_read"] = float(look.mean())  # the oracle's canonical tree search
             if name == "pairs":
                 sh = hq[sel][np.arange(hit_cap)[None, :] < rq[sel]["n_hits"][:, None]]
                 oh = np.zeros(sh.size, oracle.HIT_DTYPE)
@@ -922,7 +942,7 @@ def run_gpu(args):
         probes["l2"] = gather_probe_phase(aln, torch, dev, stream, buf_bytes=64 << 20)
         line["gather_probe"] = probes
     info = dix.info()
-    index_bytes = 2 * (info["occ_bytes"] + info["kmer_bytes"])
+    index_bytes = 2 * (info["occ_bytes"] + info["kmer_bytes"]) + derived_index_bytes(info["n"])
     use_oracle = rank == 0 and not args.no_oracle and w.text.size <= args.oracle_max_bp
     if use_oracle:
         import oracle
@@ -955,7 +975,9 @@ def run_gpu(args):
         valid = np.arange(hit_cap)[None, :] < rg["n_hits"][:, None]
         for f in ("k", "l", "aligned_len", "strand", "n_diff", "n_mm", "n_gapo", "n_gape"):
             ok = ok and np.array_equal(np.where(valid, hg[f], 0), np.where(valid, ho[f], 0))
-        line["roofline"] = roofline(float(look.mean()), n, ms_head, probes, index_bytes, args.workload)
+        line["roofline"] = roofline(seed_blocks(w.reads, out["persistent"][0]["n_hits"]), n, ms_head, probes, index_bytes,
+                                    args.workload)
+        line["roofline"]["tree_occ_lookups_per_read"] = float(look.mean())  # the oracle's canonical tree search
         line["cpu_baseline"] = {"value": cpu_v, "unit": "reads/s", "cores": threads, "kind": "oracle",
                                 "value_1thread": cpu_v1,
                                 "sample": f"{sel.size} seeded reads of the {n}-read batch, "
