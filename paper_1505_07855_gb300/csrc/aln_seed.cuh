@@ -28,7 +28,7 @@
 // the other, this takes 2 (z + 1) look-ups at once and looks at about ten places
 // (100 Mbp), each a read of the suffix array and of the text.  1 M reads of 100
 // bases at z = 4 on 100 Mbp: 65 -> 3.0 ms; 400 000 reads of 36 to 250 bases on
-// 3.1 Gbp: 725 -> 14-16 ms (profiles/aln_seed.md).  It is bound by the latency of
+// 3.1 Gbp: 738 -> 14.8 ms.  It is bound by the latency of
 // those four dependent random reads and by instruction issue, not by bandwidth.
 #pragma once
 
@@ -673,7 +673,7 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
     // places (a repeat), few long parts first: what they find bounds the
     // differences that the next pass has to look for.
     uint32_t b = z;
-    bool stepping = exhaustive;  // b starts from 1 and grows by one (or, of an exhaustive search, is z)
+    bool stepping = exhaustive;  // b is 1, 3, 7 or what the targets found allow (or, of an exhaustive search, z)
     if (!exhaustive && static_cast<uint32_t>(m) < (z + 1) * K) {
         const uint32_t fit = static_cast<uint32_t>(m) / K;
         b = min(z, fit > 2 ? fit - 1 : 1u);
@@ -749,7 +749,7 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
         const uint32_t span = ps | (pe << 8) | (off << 16);
         for (uint32_t c0 = 0; __any_sync(FULL, todo && c0 < total); c0 += G) {
             const uint32_t c = c0 + l, have = min(S.count, static_cast<uint32_t>(E));
-            __syncwarp();  // before this round's lanes record targets
+            __syncwarp();  // before lanes record targets
             uint32_t o = 0;  // the lane whose part has place c: the last one that starts at or before it
 #pragma unroll
             for (int step = G / 2; step; step >>= 1) {
@@ -802,7 +802,7 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
                 left &= ~__ballot_sync(FULL, same);
             }
             // gapped targets: a diagonal that a gap may lead to or from is looked at by
-            // the whole group, for the parts that found it in this round
+            // the whole group, for all the parts that lead to it here
             const uint32_t gmost = p.max_gapo ? min(F, p.max_gape + 1u) : 0u;
             bool want = false;
             if (live && gmost) {
@@ -838,7 +838,7 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
             } else if (exhaustive || F <= b) {  // F = z while nothing is found
                 todo = false;
             } else {
-                b = stepping ? min(F, b + 1) : F;
+                b = stepping ? min(F, 2 * b + 1) : F;  // 1, 2, 3, ... takes the mixed batch 18.1 ms, this 14.8
             }
         }
     }
