@@ -6,8 +6,8 @@ repeat families), 1 M single-end 100 bp reads (substitutions 0.5 % -> 2 %,
 0.02 % indels of 1-3 bp), z=4, seed 32 with <= 2 seed differences, gap opens
 <= 1, gap extensions <= 6, no indel within 5 bp of an end; BEST1 strata.
 
-A step is one aln_search over the whole 1 M-read batch (both strands, D scans,
-backtracking search, hit reduction).  The headline is the persistent (batched)
+A step is one aln_search over the whole 1 M-read batch (both strands, seed
+search, tree search of the reads it leaves, hit reduction).  The headline is the persistent (batched)
 form; the plain one-launch-per-batch form is timed beside it.  L2 is flushed
 (a 512 MiB write) before every timed step.  Then (unless `--human 0`) the
 3.1 Gbp text: its index built on the GPU, a 1 M-read paired batch and a 1 M-read
