@@ -138,7 +138,9 @@ int fm_index_build_gpu(const uint8_t *text, uint64_t n, const fm_build_opts *opt
                        fm_index **out);
 
 /* Write / read the index image (little-endian binary, magic "ALNFMIX4").
- * Load returns ALN_EIO on a missing, short or malformed file. */
+ * Load returns ALN_EIO on a missing, short or malformed file, and on one whose
+ * tables do not agree with its symbols (Occ counts, C, the row of $, samples and
+ * intervals inside the rows). */
 int fm_index_save(const fm_index *idx, const char *path);
 int fm_index_load(const char *path, fm_index **out);
 
