@@ -310,9 +310,11 @@ __device__ void heavy_start_one(const HeavyCtx &H, uint32_t hid, const uint2 *db
     }
 }
 
-// Blocks of the start and decide kernels: a call without heavy reads, the usual
-// one, only pays for launching them (2048 blocks, one a possible read: 3.3 us).
-constexpr uint32_t kHeavyBlocks = 152;
+// Blocks of the start and decide kernels per SM: a call without heavy reads, the
+// usual one, only pays for launching them (1.3 us with 1 block an SM, 1.4 with 4,
+// 2.1 with one a possible read, 2048), and clearing the tables of 2048 heavy reads
+// takes 41, 20 and 15 us.
+constexpr uint32_t kHeavyBlocksPerSm = 4;
 
 __global__ void aln_heavy_start_kernel(SearchParams p, const uint2 *dbp, uint32_t n_text) {
     cudaGridDependencySynchronize();
@@ -566,92 +568,86 @@ __global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_heavy
     heavy_pass<STACK_CAP, SCORE>(X, rb, p, dbp);
 }
 
-// Score-ordered result of a handed-over read from its tables (the rule of the
-// persistent search's score writer: strata S1 / S2, order (score, strand, k, l)).
-__device__ void heavy_write_score(const SearchParams &p, const HeavySlot *T, const HeavyRead *R, uint32_t n_used,
-                                  aln_read_result *res, aln_hit *hits) {
-    aln_read_result out;
-    out.c0 = out.c1 = 0;
-    out.n_hits = 0;
-    out.d_best = 255;
-    out.best_score = 255;
-    uint32_t flags = R->flags & 0xFFu;
-    uint32_t s1 = 0xFFFFFFFFu, s2 = 0xFFFFFFFFu;
-    for (uint32_t j = 0; j < 2 * kHeavySlots; j++)
-        if (T[j].id) s1 = min(s1, static_cast<uint32_t>(T[j].wkey >> 32));
-    for (uint32_t j = 0; j < 2 * kHeavySlots; j++)
-        if (T[j].id && static_cast<uint32_t>(T[j].wkey >> 32) > s1) s2 = min(s2, static_cast<uint32_t>(T[j].wkey >> 32));
-    if (n_used) {
-        unsigned long long c0 = 0, c1 = 0;
-        uint32_t dbest = 255;
-        for (uint32_t j = 0; j < 2 * kHeavySlots; j++) {
-            if (!T[j].id) continue;
-            const uint32_t sc = static_cast<uint32_t>(T[j].wkey >> 32);
-            const unsigned long long w = (T[j].id & 0xFFFFFFFFull) - (T[j].id >> 32);
-            if (sc == s1) {
-                c0 += w;
-                dbest = min(dbest, (static_cast<uint32_t>(T[j].wkey) >> 28) & 7u);
-            } else if (sc == s2) {
-                c1 += w;
-            }
-        }
-        const bool many = p.max_best && c0 > p.max_best;
-        uint32_t kept = 0;
-        for (uint32_t j = 0; j < 2 * kHeavySlots; j++) {
-            if (!T[j].id) continue;
-            const uint32_t sc = static_cast<uint32_t>(T[j].wkey >> 32);
-            if (sc == s1 || (!many && sc == s2)) kept++;
-        }
-        if (many) flags |= ALN_FLAG_MANY_BEST;
-        const uint32_t nout = min(kept, p.hit_cap);
-        if (kept > p.hit_cap) flags |= ALN_FLAG_HIT_OVERFLOW;
-        aln_hit *Hh = hits + static_cast<uint64_t>(R->r) * p.hit_cap;
-        // order (score, strand, k, l): each round takes the least entry above the previous one
-        unsigned long long prev_s = 0, prev_o = 0;
-        bool have_prev = false;
-        for (uint32_t t = 0; t < nout; t++) {
-            bool found = false;
-            unsigned long long bs = 0, bo = 0;
-            uint32_t bkey = 0;
-            for (uint32_t j = 0; j < 2 * kHeavySlots; j++) {
-                if (!T[j].id) continue;
-                const uint32_t sc = static_cast<uint32_t>(T[j].wkey >> 32);
-                if (!(sc == s1 || (!many && sc == s2))) continue;
-                const uint32_t key = static_cast<uint32_t>(T[j].wkey);
-                // (strand, k, l) as one number: strand above the 64-bit interval order
-                const unsigned long long o = T[j].id;
-                const unsigned long long ss = (static_cast<unsigned long long>(sc) << 1) | (key >> 31);
-                if (have_prev && (ss < prev_s || (ss == prev_s && o <= prev_o))) continue;
-                if (!found || ss < bs || (ss == bs && o < bo)) {
-                    found = true;
-                    bs = ss;
-                    bo = o;
-                    bkey = key;
-                }
-            }
-            aln_hit h;
-            h.k = static_cast<uint32_t>(bo >> 32);
-            h.l = static_cast<uint32_t>(bo) - 1;
-            h.aligned_len = static_cast<uint16_t>(bkey & 0xFFFFu);
-            h.strand = static_cast<uint8_t>(bkey >> 31);
-            h.n_diff = static_cast<uint8_t>((bkey >> 28) & 7u);
-            h.n_gapo = static_cast<uint8_t>((bkey >> 24) & 15u);
-            h.n_gape = static_cast<uint8_t>((bkey >> 20) & 15u);
-            h.n_mm = static_cast<uint8_t>((bkey >> 16) & 15u);
-            h.reserved = 0;
-            Hh[t] = h;
-            prev_s = bs;
-            prev_o = bo;
-            have_prev = true;
-        }
-        out.c0 = c0 > 0xFFFFFFFFull ? 0xFFFFFFFFu : static_cast<uint32_t>(c0);
-        out.c1 = c1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : static_cast<uint32_t>(c1);
-        out.d_best = static_cast<uint8_t>(dbest);
-        out.best_score = static_cast<uint8_t>(s1 > 254 ? 254 : s1);
-        out.n_hits = static_cast<uint8_t>(nout);
+// Result of a handed-over read from its tables, by the threads of a block: hits of
+// value v (diffs, at most fin, or in the score-ordered mode the score) listed in the
+// order (v, strand, k, l), counted in the strata of the least value and the one after
+// it.  A thread places a hit by the number of listed hits before it, so a read of
+// n listed hits takes n / 128 rounds over them.  (One thread, searching the 2048
+// slots for each hit in turn, took 8.9 ms for 2048 reads, a block each, and 11.4 ms
+// on 152 blocks; this takes 0.09 ms on 608.)
+__device__ void heavy_write(const SearchParams &p, const HeavySlot *T, const HeavyRead *R, uint32_t fin,
+                            aln_read_result *res, aln_hit *hits) {
+    constexpr uint32_t kSlots = 2 * kHeavySlots;
+    const bool score = p.strata == ALN_STRATA_SCORE;
+    __shared__ uint32_t s_1, s_2, s_best, s_kept;     // least value, the next one, fewest diffs at the least, hits listed
+    __shared__ unsigned long long s_c0, s_c1;         // widths at the two values
+    __shared__ uint16_t s_slot[kSlots];               // the listed hits' slots
+    auto value = [&](unsigned long long wkey) {
+        return score ? static_cast<uint32_t>(wkey >> 32) : (static_cast<uint32_t>(wkey) >> 28) & 7u;
+    };
+    if (threadIdx.x == 0) {
+        s_1 = s_2 = 0xFFFFFFFFu;
+        s_best = 255;
+        s_kept = 0;
+        s_c0 = s_c1 = 0;
     }
-    out.flags = static_cast<uint8_t>(flags);
-    res[R->r] = out;
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < kSlots; j += blockDim.x)
+        if (T[j].id && (score || value(T[j].wkey) <= fin)) atomicMin(&s_1, value(T[j].wkey));
+    __syncthreads();
+    if (score) {
+        for (uint32_t j = threadIdx.x; j < kSlots; j += blockDim.x)
+            if (T[j].id && value(T[j].wkey) > s_1) atomicMin(&s_2, value(T[j].wkey));
+    } else if (threadIdx.x == 0 && s_1 < fin) {
+        s_2 = s_1 + 1;
+    }
+    __syncthreads();
+    const uint32_t v1 = s_1, v2 = s_2;
+    for (uint32_t j = threadIdx.x; j < kSlots; j += blockDim.x) {
+        if (!T[j].id) continue;
+        const uint32_t v = value(T[j].wkey);
+        const unsigned long long w = (T[j].id & 0xFFFFFFFFull) - (T[j].id >> 32);
+        if (v == v1) {
+            atomicAdd(&s_c0, w);
+            atomicMin(&s_best, (static_cast<uint32_t>(T[j].wkey) >> 28) & 7u);
+        } else if (v == v2) {
+            atomicAdd(&s_c1, w);
+        }
+    }
+    __syncthreads();
+    const bool many = score && p.max_best && s_c0 > p.max_best;
+    for (uint32_t j = threadIdx.x; j < kSlots; j += blockDim.x) {
+        if (!T[j].id) continue;
+        const uint32_t v = value(T[j].wkey);
+        if (score ? v == v1 || (!many && v == v2) : v <= fin) s_slot[atomicAdd(&s_kept, 1u)] = static_cast<uint16_t>(j);
+    }
+    __syncthreads();
+    const uint32_t kept = s_kept, nout = min(kept, p.hit_cap);
+    for (uint32_t i = threadIdx.x; i < kept; i += blockDim.x) {
+        const HeavySlot e = T[s_slot[i]];
+        const uint32_t key = static_cast<uint32_t>(e.wkey), o = (value(e.wkey) << 1) | (key >> 31);
+        uint32_t before = 0;
+        for (uint32_t j = 0; j < kept && before < nout; j++) {
+            const HeavySlot f = T[s_slot[j]];
+            const uint32_t fo = (value(f.wkey) << 1) | (static_cast<uint32_t>(f.wkey) >> 31);
+            before += fo < o || (fo == o && f.id < e.id) ? 1u : 0u;
+        }
+        if (before < nout)
+            put_hit(hits + static_cast<uint64_t>(R->r) * p.hit_cap + before, static_cast<uint32_t>(e.id >> 32),
+                    static_cast<uint32_t>(e.id) - 1u, key);
+    }
+    if (threadIdx.x == 0) {
+        const bool any = kept > 0;
+        aln_read_result out;
+        out.c0 = static_cast<uint32_t>(min(any ? s_c0 : 0ull, 0xFFFFFFFFull));
+        out.c1 = static_cast<uint32_t>(min(any ? s_c1 : 0ull, 0xFFFFFFFFull));
+        out.d_best = static_cast<uint8_t>(any ? s_best : 255u);
+        out.best_score = static_cast<uint8_t>(score ? (any ? min(v1, 254u) : 255u) : 0u);
+        out.n_hits = static_cast<uint8_t>(nout);
+        out.flags = static_cast<uint8_t>((R->flags & 0xFFu) | (many ? ALN_FLAG_MANY_BEST : 0u) |
+                                         (kept > p.hit_cap ? ALN_FLAG_HIT_OVERFLOW : 0u));
+        res[R->r] = out;
+    }
 }
 
 // One block per handed-over read after a pass: the iterative deepening rule on
@@ -715,88 +711,8 @@ __device__ void heavy_decide_one(const SearchParams &p, uint32_t hid, const uint
         }
         return;
     }
-    if (threadIdx.x != 0) return;
-    if (p.strata == ALN_STRATA_SCORE) {
-        heavy_write_score(p, T, R, s_n, res, hits);
-        R->state = 1;
-        return;
-    }
-    // the result: hits with diffs <= the final budget, ordered (diffs, strand, k, l)
-    const uint32_t fin = s_final;
-    aln_read_result out;
-    out.c0 = out.c1 = 0;
-    out.n_hits = 0;
-    out.d_best = 255;
-    out.best_score = 0;
-    uint32_t dbest = 255;
-    for (uint32_t j = 0; j < 2 * kHeavySlots; j++)
-        if (T[j].id && ((static_cast<uint32_t>(T[j].wkey) >> 28) & 7u) <= fin) dbest = min(dbest, (static_cast<uint32_t>(T[j].wkey) >> 28) & 7u);
-    uint32_t flags = R->flags & 0xFFu;
-    if (dbest != 255 && s_n) {
-        unsigned long long c0 = 0, c1 = 0;
-        uint32_t kept = 0;
-        for (uint32_t j = 0; j < 2 * kHeavySlots; j++) {
-            if (!T[j].id) continue;
-            const uint32_t d = (static_cast<uint32_t>(T[j].wkey) >> 28) & 7u;
-            if (d > fin) continue;
-            kept++;
-            const unsigned long long w = (T[j].id & 0xFFFFFFFFull) - (T[j].id >> 32);
-            if (d == dbest) c0 += w;
-            else if (d == dbest + 1) c1 += w;
-        }
-        out.c0 = c0 > 0xFFFFFFFFull ? 0xFFFFFFFFu : static_cast<uint32_t>(c0);
-        out.c1 = c1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : static_cast<uint32_t>(c1);
-        out.d_best = static_cast<uint8_t>(dbest);
-        const uint32_t nout = min(kept, p.hit_cap);
-        if (kept > p.hit_cap) flags |= ALN_FLAG_HIT_OVERFLOW;
-        aln_hit *Hh = hits + static_cast<uint64_t>(R->r) * p.hit_cap;
-        // selection of the nout smallest by (diffs, strand, k, l): each round takes
-        // the least entry above the previous one
-        uint32_t pk = 0, pl = 0, pkey = 0;
-        bool have_prev = false;
-        for (uint32_t t = 0; t < nout; t++) {
-            bool found = false;
-            uint32_t bk = 0, bl = 0, bkey = 0;
-            for (uint32_t j = 0; j < 2 * kHeavySlots; j++) {
-                if (!T[j].id) continue;
-                const uint32_t key = static_cast<uint32_t>(T[j].wkey);
-                const uint32_t d = (key >> 28) & 7u;
-                if (d > fin) continue;
-                const uint32_t k = static_cast<uint32_t>(T[j].id >> 32), l = static_cast<uint32_t>(T[j].id);
-                const uint32_t o = (d << 1) | (key >> 31);
-                if (have_prev) {
-                    const uint32_t po = (((pkey >> 28) & 7u) << 1) | (pkey >> 31);
-                    if (o < po || (o == po && (k < pk || (k == pk && l <= pl)))) continue;
-                }
-                if (!found) {
-                    found = true;
-                    bk = k; bl = l; bkey = key;
-                } else {
-                    const uint32_t bo = (((bkey >> 28) & 7u) << 1) | (bkey >> 31);
-                    if (o < bo || (o == bo && (k < bk || (k == bk && l < bl)))) {
-                        bk = k; bl = l; bkey = key;
-                    }
-                }
-            }
-            aln_hit h;
-            h.k = bk;
-            h.l = bl - 1;
-            h.aligned_len = static_cast<uint16_t>(bkey & 0xFFFFu);
-            h.strand = static_cast<uint8_t>(bkey >> 31);
-            h.n_diff = static_cast<uint8_t>((bkey >> 28) & 7u);
-            h.n_gapo = static_cast<uint8_t>((bkey >> 24) & 15u);
-            h.n_gape = static_cast<uint8_t>((bkey >> 20) & 15u);
-            h.n_mm = static_cast<uint8_t>((bkey >> 16) & 15u);
-            h.reserved = 0;
-            Hh[t] = h;
-            pk = bk; pl = bl; pkey = bkey;
-            have_prev = true;
-        }
-        out.n_hits = static_cast<uint8_t>(nout);
-    }
-    out.flags = static_cast<uint8_t>(flags);
-    res[R->r] = out;
-    R->state = 1;
+    heavy_write(p, T, R, s_final, res, hits);
+    if (threadIdx.x == 0) R->state = 1;
 }
 
 __global__ void aln_heavy_decide_kernel(SearchParams p, const uint2 *dbp, uint32_t n_text, aln_read_result *res,
@@ -1129,11 +1045,12 @@ static cudaError_t launch_cap(const DIndex &X, const ReadBatch &rb, uint32_t n, 
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&hb, aln_heavy_pass_kernel<CAP, SCORE>, kThreads, 0);
             // the ring holds at most 2 entries per thread of the grid (the pass kernel's low-water mark)
             const unsigned hgrid = min(static_cast<unsigned>(sms * (hb > 0 ? hb : 1)), kHeavyPool / (2u * kThreads));
-            e = launch_after(aln_heavy_start_kernel, kHeavyBlocks, st, nullptr, pp, dbp, X.t[0].n);
+            const unsigned hblocks = min(kHeavyReads, static_cast<uint32_t>(sms) * kHeavyBlocksPerSm);
+            e = launch_after(aln_heavy_start_kernel, hblocks, st, nullptr, pp, dbp, X.t[0].n);
             for (uint32_t pass = 0; pass < kHeavyPasses && e == cudaSuccess; pass++) {
                 e = launch_after(aln_heavy_pass_kernel<CAP, SCORE>, hgrid, st, nullptr, X, rb, pp, dbp);
                 if (e == cudaSuccess)
-                    e = launch_after(aln_heavy_decide_kernel, kHeavyBlocks, st, nullptr, pp, dbp, X.t[0].n, res, hits,
+                    e = launch_after(aln_heavy_decide_kernel, hblocks, st, nullptr, pp, dbp, X.t[0].n, res, hits,
                                      pass + 1 == kHeavyPasses ? 1 : 0);
             }
             if (e != cudaSuccess) return e;
