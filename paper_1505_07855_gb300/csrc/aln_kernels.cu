@@ -64,48 +64,46 @@ __global__ void __launch_bounds__(kThreads) aln_plain_kernel(DIndex X, ReadBatch
     plain_tree<STACK_CAP>(X, rb, p, r, s_bases + threadIdx.x, s_nmask + threadIdx.x, res, hits);
 }
 
-// The same after a seed search: the block answers what it can of its reads,
-// kPlainLanes lanes a read, and its first threads search the rest.  A block takes
-// a quarter of its threads' number of reads, so that a batch of few reads still has
-// blocks for every SM.  The tree search is out of line, or its registers would
-// leave room for three blocks on an SM (100 000 reads of 100 bases on 100 Mbp: 1.47 ms
-// in one kernel with it, 0.47 ms so; the tree search alone takes 52 ms).
-constexpr int kPlainLanes = 16;
-constexpr uint32_t kPlainReads = kThreads / 4;
+// The same after a seed search: a warp answers what it can of its reads (at most 32),
+// kPlainLanes lanes a read, and then searches the trees of the others, a lane each,
+// on its own, so that some warps search trees while others look up seeds.  It takes
+// as many reads as fill the device once, up to 32: a batch of nothing but repeats
+// then has as many trees in flight, and as full warps, as without the seed search.
+// 400 000 reads of 60 bases out of 30 000 copies take 70.6 ms and 100 000 23.1, where
+// blocks of 32 reads whose first threads searched the rest took 112 and 34 and the
+// tree search alone takes 66.6 and 24.0; 100 000 reads of 100 bases on 100 Mbp, next
+// to none of them left, 0.455 ms (0.475, and 52).  Resident blocks an SM: 5 / 6 / 7 /
+// 8 take 76.5 / 70.6 / 69.2 / 70.2 and 27.8 / 23.1 / 25.9 / 27.7 ms for the copies,
+// 0.571 / 0.455 / 0.452 / 0.434 for the others.
+#ifndef ALN_PLAIN_BLOCKS
+#define ALN_PLAIN_BLOCKS 6
+#endif
+constexpr int kPlainLanes = 16, kPlainBlocks = ALN_PLAIN_BLOCKS;
+constexpr uint32_t kPlainStep = 32 / kPlainLanes;  // reads a warp takes at once
 constexpr uint32_t kPlainTargets = 32, kPlainPlaces = 2048;
 
 template <int STACK_CAP>
-__device__ __noinline__ void plain_rest(const DIndex &X, const ReadBatch &rb, const SearchParams &p, uint32_t r,
-                                        uint32_t *sb, uint32_t *sn, aln_read_result *res, aln_hit *hits) {
-    plain_tree<STACK_CAP>(X, rb, p, r, sb, sn, res, hits);
-}
-
-template <int STACK_CAP>
-__global__ void __launch_bounds__(kThreads, 5) aln_plain_seed_kernel(const __grid_constant__ DIndex X,
-                                                                     const __grid_constant__ ReadBatch rb,
-                                                                     uint32_t n_reads,
-                                                                     const __grid_constant__ SearchParams p,
-                                                                     aln_read_result *res, aln_hit *hits) {
-    __shared__ union {
-        SeedRead<kPlainTargets> read[kThreads / kPlainLanes];
-        struct {
-            uint32_t bases[kReadWords * kThreads], nmask[kMaskWords * kThreads];
-        } tree;
-    } sh;
-    __shared__ uint32_t s_rest[kPlainReads], s_count;
-    if (threadIdx.x == 0) s_count = 0;
-    __syncthreads();
-    const uint32_t group = threadIdx.x / kPlainLanes, first = blockIdx.x * kPlainReads;
-    for (uint32_t i = group; i < kPlainReads; i += kThreads / kPlainLanes) {  // the same rounds for every group
-        const bool active = first + i < n_reads;
-        const bool done = seed_search<kPlainLanes, kPlainTargets, false, true>(X, rb, p, sh.read[group], first + i, active,
-                                                                         kPlainPlaces, res, hits);
-        if (active && !done && threadIdx.x % kPlainLanes == 0) s_rest[atomicAdd(&s_count, 1u)] = first + i;
+__global__ void __launch_bounds__(kThreads, kPlainBlocks) aln_plain_seed_kernel(
+    const __grid_constant__ DIndex X, const __grid_constant__ ReadBatch rb, uint32_t n_reads, uint32_t warp_reads,
+    const __grid_constant__ SearchParams p, aln_read_result *res, aln_hit *hits) {
+    __shared__ SeedRead<kPlainTargets> s_read[kThreads / kPlainLanes];
+    __shared__ uint32_t s_bases[kReadWords * kThreads], s_nmask[kMaskWords * kThreads], s_rest[kThreads];
+    const uint32_t group = threadIdx.x / kPlainLanes, lane = threadIdx.x & 31u, col = threadIdx.x & ~31u;
+    const uint64_t first = (static_cast<uint64_t>(blockIdx.x) * (kThreads / 32) + threadIdx.x / 32) * warp_reads;
+    uint32_t left = 0;  // reads in the warp's part of s_rest
+    for (uint32_t t = 0; t < warp_reads && first + t < n_reads; t += kPlainStep) {
+        const uint64_t r = first + t + group % kPlainStep;
+        const bool active = t + group % kPlainStep < warp_reads && r < n_reads;
+        const bool done = seed_search<kPlainLanes, kPlainTargets, false, true>(
+            X, rb, p, s_read[group], static_cast<uint32_t>(r), active, kPlainPlaces, res, hits);
+        const bool rest = active && !done && threadIdx.x % kPlainLanes == 0;
+        const unsigned all = __ballot_sync(0xFFFFFFFFu, rest);
+        if (rest) s_rest[col + left + __popc(all & ((1u << lane) - 1u))] = static_cast<uint32_t>(r);
+        left += __popc(all);
     }
-    __syncthreads();
-    if (threadIdx.x < s_count)
-        plain_rest<STACK_CAP>(X, rb, p, s_rest[threadIdx.x], sh.tree.bases + threadIdx.x, sh.tree.nmask + threadIdx.x,
-                              res, hits);
+    __syncwarp();
+    if (lane < left)
+        plain_tree<STACK_CAP>(X, rb, p, s_rest[threadIdx.x], s_bases + threadIdx.x, s_nmask + threadIdx.x, res, hits);
 }
 
 #ifndef ALN_PERSISTENT_MIN_BLOCKS
@@ -963,15 +961,19 @@ template <int CAP, int SMEM, bool SCORE>
 static cudaError_t launch_cap(const DIndex &X, const ReadBatch &rb, uint32_t n, const SearchParams &p,
                               aln_read_result *res, aln_hit *hits, uint32_t mode, uint32_t *queue,
                               void *scratch, cudaStream_t st) {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (mode == ALN_MODE_PLAIN) {
-        if (seed_supported(X, p))
-            aln_plain_seed_kernel<CAP><<<(n + kPlainReads - 1) / kPlainReads, kThreads, 0, st>>>(X, rb, n, p, res, hits);
-        else
+        if (seed_supported(X, p)) {
+            const uint32_t warps = static_cast<uint32_t>(sms) * kPlainBlocks * (kThreads / 32);
+            const uint32_t each = n <= warps ? 1u : min(32u, kPlainStep * (n / (kPlainStep * warps) + 1u));
+            const uint32_t block = each * (kThreads / 32);
+            aln_plain_seed_kernel<CAP><<<n / block + (n % block ? 1u : 0u), kThreads, 0, st>>>(X, rb, n, each, p, res, hits);
+        } else {
             aln_plain_kernel<CAP><<<(n + kThreads - 1) / kThreads, kThreads, 0, st>>>(X, rb, n, p, res, hits);
+        }
     } else {
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, aln_persistent_kernel<CAP, SMEM, SCORE>, kThreads, 0);
         if (p.blocks_per_sm && static_cast<int>(p.blocks_per_sm) < per_sm) per_sm = p.blocks_per_sm;
         if (per_sm < 1) per_sm = 1;
