@@ -94,9 +94,9 @@ __global__ void __launch_bounds__(kThreads, kPlainBlocks) aln_plain_seed_kernel(
     for (uint32_t t = 0; t < warp_reads && first + t < n_reads; t += kPlainStep) {
         const uint64_t r = first + t + group % kPlainStep;
         const bool active = t + group % kPlainStep < warp_reads && r < n_reads;
-        const bool done = seed_search<kPlainLanes, kPlainTargets, false, true>(
+        const SeedAnswer got = seed_search<kPlainLanes, kPlainTargets, false, true>(
             X, rb, p, s_read[group], static_cast<uint32_t>(r), active, kPlainPlaces, res, hits);
-        const bool rest = active && !done && threadIdx.x % kPlainLanes == 0;
+        const bool rest = active && got != kSeedDone && threadIdx.x % kPlainLanes == 0;
         const unsigned all = __ballot_sync(0xFFFFFFFFu, rest);
         if (rest) s_rest[col + left + __popc(all & ((1u << lane) - 1u))] = static_cast<uint32_t>(r);
         left += __popc(all);
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(kThreads) aln_dscan_kernel(DIndex X, ReadBatch
 // ---------------------------------------------------------------- seed search
 //
 // aln_seed_kernel answers the reads whose parts lead to few places (see
-// aln_seed.cuh), G lanes a read; aln_seed_wide_kernel takes the reads it leaves,
+// aln_seed.cuh), G lanes a read; aln_seed_wide_kernel takes the reads it leaves for more lanes,
 // a warp each with room for kCandCap targets; aln_dscan_list_kernel scans the D
 // arrays of what is left then, which the persistent search and the heavy phase
 // search as before: the rest fills the visit order from its end, and the queue
@@ -805,14 +805,12 @@ struct SeedCounts {          // in the scratch's first words, cleared before the
 // Room for targets and places to look at, first for a read's 8 or 16 lanes: past
 // that the other reads of the warp wait for it, so it goes to a warp of its own
 // (300 000 mates on 3.1 Gbp: 8.4 / 7.15 / 6.2 ms with 1024 / 256 / 64 places).
-// There, kCandCap targets are what the tree search keeps, and 16384 places are half
-// a millisecond of a warp, about what the tree search of such a read costs.
+// There, kCandCap targets are what the tree search keeps.
 constexpr uint32_t kSeedTargets = 32;
 #ifndef ALN_SEED_PLACES
 #define ALN_SEED_PLACES 64
 #endif
 constexpr uint32_t kSeedPlaces = ALN_SEED_PLACES;
-constexpr uint32_t kWidePlaces = 16384;
 
 // Resident blocks per SM: 4 / 5 / 6 take 3.36 / 3.08 / 2.98 ms for 1 M reads of 100
 // bases on 100 Mbp and 6.28 / 5.87 / 5.76 ms for 300 000 mates on 3.1 Gbp (latency; 6
@@ -827,7 +825,7 @@ constexpr uint32_t kWidePlaces = 16384;
 template <int G, bool SCORE>
 __global__ void __launch_bounds__(kThreads, ALN_SEED_MIN_BLOCKS) aln_seed_kernel(const __grid_constant__ DIndex X, ReadBatch rb, uint32_t n, const __grid_constant__ SearchParams p,
                                                             aln_read_result *res, aln_hit *hits, SeedCounts *counts,
-                                                            uint32_t *wide) {
+                                                            uint32_t *wide, uint32_t *order_end) {
     __shared__ SeedRead<kSeedTargets> s_read[kThreads / G];
     if (blockIdx.x == 0) {  // what the later kernels report and count in
         if (p.status && threadIdx.x == 0) *p.status = 0;
@@ -836,9 +834,12 @@ __global__ void __launch_bounds__(kThreads, ALN_SEED_MIN_BLOCKS) aln_seed_kernel
     }
     const uint64_t r = (static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x) / G;
     const bool active = r < n;
-    const bool done = seed_search<G, kSeedTargets, SCORE>(X, rb, p, s_read[threadIdx.x / G], static_cast<uint32_t>(r),
-                                                          active, kSeedPlaces, res, hits);
-    if (active && !done && (threadIdx.x & (G - 1)) == 0) wide[atomicAdd(&counts->wide, 1u)] = static_cast<uint32_t>(r);
+    const SeedAnswer got = seed_search<G, kSeedTargets, SCORE>(X, rb, p, s_read[threadIdx.x / G],
+                                                               static_cast<uint32_t>(r), active, kSeedPlaces, res, hits);
+    if (active && got != kSeedDone && (threadIdx.x & (G - 1)) == 0) {
+        if (got == kSeedTree) *(order_end - 1 - atomicAdd(&counts->rest, 1u)) = static_cast<uint32_t>(r);
+        else wide[atomicAdd(&counts->wide, 1u)] = static_cast<uint32_t>(r);
+    }
 }
 
 template <bool SCORE>
@@ -855,9 +856,9 @@ __global__ void __launch_bounds__(kThreads, ALN_WIDE_MIN_BLOCKS) aln_seed_wide_k
         i = __shfl_sync(0xFFFFFFFFu, i, 0);
         if (i >= n) break;
         const uint32_t r = wide[i];
-        const bool done = seed_search<32, kCandCap, SCORE>(X, rb, p, s_read[threadIdx.x / 32], r, true, kWidePlaces, res,
-                                                           hits);
-        if (!done && lane == 0) *(order_end - 1 - atomicAdd(&counts->rest, 1u)) = r;
+        const SeedAnswer got = seed_search<32, kCandCap, SCORE>(X, rb, p, s_read[threadIdx.x / 32], r, true, kWidePlaces,
+                                                                res, hits);
+        if (got != kSeedDone && lane == 0) *(order_end - 1 - atomicAdd(&counts->rest, 1u)) = r;
     }
 }
 
@@ -996,10 +997,10 @@ static cudaError_t launch_cap(const DIndex &X, const ReadBatch &rb, uint32_t n, 
             // parts of both strands on 8 lanes for z <= 3, else on 16
             if (p.z <= 3)
                 aln_seed_kernel<8, SCORE><<<static_cast<unsigned>((8ull * n + kThreads - 1) / kThreads), kThreads, 0, st>>>(
-                    X, rb, n, pp, res, hits, counts, wide);
+                    X, rb, n, pp, res, hits, counts, wide, order + n);
             else
                 aln_seed_kernel<16, SCORE><<<static_cast<unsigned>((16ull * n + kThreads - 1) / kThreads), kThreads, 0, st>>>(
-                    X, rb, n, pp, res, hits, counts, wide);
+                    X, rb, n, pp, res, hits, counts, wide, order + n);
             const uint32_t wb = min((n + 3u) / 4u, static_cast<uint32_t>(sms) * 6u);
             cudaError_t e = launch_after(aln_seed_wide_kernel<SCORE>, wb, st, nullptr, X, rb, pp, res, hits, counts, wide,
                                          order + n);

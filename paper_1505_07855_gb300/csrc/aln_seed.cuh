@@ -580,14 +580,24 @@ __device__ __noinline__ bool reduce_targets(const DIndex &X, const SearchParams 
     return write;
 }
 
+// What became of a read: its result is written; it has too many places or targets
+// for this group (nothing is written then); or more places than a group of a whole
+// warp takes, so that only the tree search is left.  Told apart, reads of the
+// third kind save the wide kernel's try: 400 000 reads of 60 bases out of 30 000 copies
+// take 33.4 ms, not 37.9 (the tree search alone 30.2), 100 000 of one letter 4.18, not
+// 5.09 (4.18).
+enum SeedAnswer : uint32_t { kSeedDone, kSeedWide, kSeedTree };
+
+// The most places a read's search looks at.  16384 are half a millisecond of a warp,
+// about what the tree search of such a read costs.
+constexpr uint32_t kWidePlaces = 16384;
+
 // Search of one read by the G lanes of a group; all 32 lanes of the warp call it
-// together (other groups with their own reads, or with active = false).  True
-// if the read's result was written; false if it has too many places or targets
-// for this form (nothing is written then).  CALL: the gapped stage out of line
+// together (other groups with their own reads, or with active = false).  CALL: the gapped stage out of line
 // (1 M reads take 3.37 ms with it and 2.93 without; in the plain kernel, whose tree
 // search takes its registers, 100 000 take 0.48 ms with it and 1.25 without).
 template <int G, int E, bool SCORE, bool CALL = false>
-__device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchParams &p, SeedRead<E> &S, uint32_t r,
+__device__ SeedAnswer seed_search(const DIndex &X, const ReadBatch &rb, const SearchParams &p, SeedRead<E> &S, uint32_t r,
                             bool active, uint32_t max_places, aln_read_result *res, aln_hit *hits) {
     constexpr unsigned FULL = 0xFFFFFFFFu;
     constexpr uint32_t kHalf = G / 2;
@@ -680,7 +690,8 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
     }
     uint32_t F = z;            // differences a target may still have
     uint32_t dmin = 255;       // fewest found
-    bool todo = search, failed = false;
+    bool todo = search;
+    SeedAnswer failed = kSeedDone;
     while (__any_sync(FULL, todo)) {
         // the rows of this lane's part
         uint32_t lo = 0, hi = 0, width = 0, ps = 0, pe = 0, off = 0;  // part [ps, pe) and first matched base, in pattern order
@@ -743,7 +754,7 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
             stepping = true;
             total = 0;
         } else if (todo && total > max_places) {
-            failed = true;
+            failed = total > kWidePlaces ? kSeedTree : kSeedWide;
             todo = false;
         }
         const uint32_t span = ps | (pe << 8) | (off << 16);
@@ -831,7 +842,7 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
         }
         if (todo) {
             if (S.count > static_cast<uint32_t>(E)) {
-                failed = true;
+                failed = kSeedWide;
                 todo = false;
             } else if (again) {
                 b = 1;
@@ -864,11 +875,11 @@ __device__ bool seed_search(const DIndex &X, const ReadBatch &rb, const SearchPa
         } else if (l == 0 && answer) {
             empty_result<SCORE>(res + r, flags);
         }
-        return (search && !failed) || answer;
+        return failed;
     }
     const bool written = reduce_targets<G, E, SCORE>(X, p, S, r, cnt, F, search && !failed, group_lanes, res, hits);
     if (answer && l == 0) empty_result<SCORE>(res + r, flags);
-    return written || answer;
+    return failed ? failed : (search && !written ? kSeedWide : kSeedDone);
 }
 
 }  // namespace aln
