@@ -336,8 +336,8 @@ uint64_t aln_search_scratch_bytes(uint32_t n_reads);
  * tail says little about a batch's, and lanes that help a read early keep its
  * owner's expansions below heavy_after, so that it never reaches the heavy
  * phase).  The choice
- * is cached per (index, sample size, sample z array, limits): a repeated call
- * returns it without timing.  Blocks on stream.  ALN_EINVAL for an empty
+ * is cached per (index, sample size, sample z array, limits, help_after,
+ * heavy_after, l2_window): a repeated call returns it without timing.  Blocks on stream.  ALN_EINVAL for an empty
  * sample. */
 int aln_autotune(const fm_dindex *idx, const aln_batch *sample, uint32_t n_reads, aln_params *params,
                  aln_result *scratch, void *stream, float *best_ms);

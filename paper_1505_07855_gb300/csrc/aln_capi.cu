@@ -313,12 +313,13 @@ extern "C" int aln_search(const fm_dindex *idx, const aln_batch *batch, uint32_t
 // ---------------------------------------------------------------- autotuner
 
 namespace {
-// Autotuner choices, cached per (index, sample size, limits).
+// Autotuner choices, cached per (index, sample size, limits): everything that
+// selects the search (a work or loop limit is the tree search's) or its schedule.
 struct TuneKey {
     const fm_dindex *idx;
     uint32_t n;
     uint8_t z, gapo, gape, seed_len, seed_z, e, hit_cap, strata;
-    uint32_t work_limit;
+    uint32_t work_limit, loop_limit, heavy_after, help_after, l2_window;
     const void *zarr;
     bool operator==(const TuneKey &o) const { return std::memcmp(this, &o, sizeof(TuneKey)) == 0; }
 };
@@ -350,7 +351,8 @@ extern "C" int aln_autotune(const fm_dindex *idx, const aln_batch *sample, uint3
     key.z = params->z; key.gapo = params->max_gapo; key.gape = params->max_gape;
     key.seed_len = params->seed_len; key.seed_z = params->seed_z; key.e = params->indel_end_skip;
     key.hit_cap = params->hit_cap; key.strata = params->strata;
-    key.work_limit = params->work_limit;
+    key.work_limit = params->work_limit; key.loop_limit = params->loop_limit;
+    key.heavy_after = params->heavy_after; key.help_after = params->help_after; key.l2_window = params->l2_window;
     key.zarr = sample->z ? static_cast<const void *>(sample->z) : nullptr;
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
