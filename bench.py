@@ -394,15 +394,6 @@ def seed_blocks(reads, n_hits):
     return float(2 * (reads.z.astype(np.float64).mean() + 1) + n_hits.astype(np.float64).mean() * (2 + text))
 
 
-def derived_index_bytes(n):
-    """Bytes of the arrays the upload derives from an index of n bases (aln_derive.cu):
-    both suffix arrays, a quarter of their inverses, the text's planes, the k-mer table."""
-    k = 1
-    while k < 16 and 4 ** (k + 1) <= 4 * (n + 1):
-        k += 1
-    return 8 * n + 2 * n + n // 4 + 4 * 4 ** k
-
-
 def roofline(lookups_per_read, n, ms, probes, index_bytes, workload_name):
     """Achieved algorithmic bytes/s of the search (64 B per random block read it
     cannot do without: seed_blocks) against the random 64-byte gather rate of the
@@ -572,7 +563,7 @@ def human_phase(args, aln, torch, dev, stream, flush):
     out["index_build"] = {"where": "gpu (fm_index_build_gpu)", "s": time.time() - t0}
     dix = hix.to_device(dev.index)
     info = dix.info()
-    index_bytes = 2 * (info["occ_bytes"] + info["kmer_bytes"]) + derived_index_bytes(info["n"])
+    index_bytes = 2 * (info["occ_bytes"] + info["kmer_bytes"]) + dix.derived_bytes()
     del hix
     al = aln.Aligner(dix)
     hit_cap = 32
@@ -943,7 +934,7 @@ def run_gpu(args):
         probes["l2"] = gather_probe_phase(aln, torch, dev, stream, buf_bytes=64 << 20)
         line["gather_probe"] = probes
     info = dix.info()
-    index_bytes = 2 * (info["occ_bytes"] + info["kmer_bytes"]) + derived_index_bytes(info["n"])
+    index_bytes = 2 * (info["occ_bytes"] + info["kmer_bytes"]) + dix.derived_bytes()
     use_oracle = rank == 0 and not args.no_oracle and w.text.size <= args.oracle_max_bp
     if use_oracle:
         import oracle

@@ -78,10 +78,12 @@ class Index:
         check(lib().fm_index_info(self._h, ctypes.byref(i)), "fm_index_info")
         return _info_dict(i)
 
-    def to_device(self, device: int = 0, stream=None) -> "DeviceIndex":
+    def to_device(self, device: int = 0, stream=None, derived: bool = True) -> "DeviceIndex":
+        """The index on a device; derived=False uploads the image alone
+        (fm_index_to_device_image), for less memory and slower searches."""
+        upload = lib().fm_index_to_device if derived else lib().fm_index_to_device_image
         out = ctypes.c_void_p()
-        check(lib().fm_index_to_device(self._h, device, _stream_ptr(stream), ctypes.byref(out)),
-              "fm_index_to_device")
+        check(upload(self._h, device, _stream_ptr(stream), ctypes.byref(out)), "fm_index_to_device")
         return DeviceIndex(out.value, device)
 
     def __del__(self):
@@ -116,6 +118,10 @@ class DeviceIndex:
         i = _lib.fm_index_info_t()
         check(lib().fm_dindex_info(self._h, ctypes.byref(i)), "fm_dindex_info")
         return _info_dict(i)
+
+    def derived_bytes(self) -> int:
+        """Bytes of the arrays derived at upload; 0 = served from the image alone."""
+        return int(lib().fm_dindex_derived_bytes(self._h))
 
     def search(self, bases, nmask, offsets, lens, z, n_reads: int, params: "Params",
                res_out, hits_out, stream=None, status=None, scratch=None) -> None:

@@ -118,6 +118,8 @@ SIGNATURES = {
     "fm_index_save": (ctypes.c_int, [P, ctypes.c_char_p]),
     "fm_index_load": (ctypes.c_int, [ctypes.c_char_p, ctypes.POINTER(P)]),
     "fm_index_to_device": (ctypes.c_int, [P, ctypes.c_int, P, ctypes.POINTER(P)]),
+    "fm_index_to_device_image": (ctypes.c_int, [P, ctypes.c_int, P, ctypes.POINTER(P)]),
+    "fm_dindex_derived_bytes": (ctypes.c_uint64, [P]),
     "fm_dindex_free": (None, [P]),
     "fm_dindex_info": (ctypes.c_int, [P, ctypes.POINTER(fm_index_info_t)]),
     "aln_search": (ctypes.c_int, [P, ctypes.POINTER(aln_batch), ctypes.c_uint32,

@@ -41,6 +41,7 @@ struct fm_dindex {
     std::atomic<uint32_t> next_capture{0};
     cudaMemPool_t pool = nullptr;         // stream-ordered per-call scratch (D pre-pass, visit order)
     void *derived = nullptr;              // arrays derived from the image (aln_derive.cu), one buffer
+    uint64_t derived_bytes = 0;
 };
 
 // Search parameters from the ABI struct; ALN_OK or ALN_EINVAL with a message.
@@ -109,7 +110,7 @@ extern "C" void fm_dindex_free(fm_dindex *d) {
     delete d;
 }
 
-extern "C" int fm_index_to_device(const fm_index *idx, int device, void *stream, fm_dindex **out) {
+static int to_device(const fm_index *idx, int device, void *stream, bool with_derived, fm_dindex **out) {
     if (!idx || !out) return fail(ALN_EINVAL, "fm_index_to_device: null argument");
     *out = nullptr;
     int ndev = 0;
@@ -180,7 +181,7 @@ extern "C" int fm_index_to_device(const fm_index *idx, int device, void *stream,
             d->pool = nullptr;
         }
     }
-    if (rc == ALN_OK) {  // optional: without the derived arrays every call works from the image
+    if (rc == ALN_OK && with_derived) {  // optional: without the derived arrays every call works from the image
         size_t free_b = 0, total_b = 0;
         const uint64_t want = derived_bytes(d->info.n);
         bool ok = false;
@@ -188,6 +189,7 @@ extern "C" int fm_index_to_device(const fm_index *idx, int device, void *stream,
             cudaMalloc(&d->derived, want) == cudaSuccess)
             e = derive(d->X, d->derived, st, &ok);
         cudaGetLastError();  // a failed allocation is no error of the call
+        if (ok) d->derived_bytes = want;
         if (d->derived && !ok) {
             cudaFree(d->derived);
             d->derived = nullptr;
@@ -202,6 +204,16 @@ extern "C" int fm_index_to_device(const fm_index *idx, int device, void *stream,
     *out = d;
     return ALN_OK;
 }
+
+extern "C" int fm_index_to_device(const fm_index *idx, int device, void *stream, fm_dindex **out) {
+    return to_device(idx, device, stream, true, out);
+}
+
+extern "C" int fm_index_to_device_image(const fm_index *idx, int device, void *stream, fm_dindex **out) {
+    return to_device(idx, device, stream, false, out);
+}
+
+extern "C" uint64_t fm_dindex_derived_bytes(const fm_dindex *d) { return d ? d->derived_bytes : 0; }
 
 extern "C" int fm_dindex_info(const fm_dindex *d, fm_index_info_t *info) {
     if (!d || !info) return fail(ALN_EINVAL, "fm_dindex_info: null argument");
