@@ -33,17 +33,14 @@ sys.path.insert(0, ROOT)
 
 METRIC = "reads/s bit-exact vs oracle (batched vs plain, 1 GB300); % HBM roofline; p99 ms"
 BYTES_PER_LOOKUP = 64
-# DRAM bytes (read + write) of the seed search's kernels per read from one ncu
-# capture of each workload (a few hundred thousand reads, scaled per read; the
-# profile summaries under profiles/ give the command).  Used only while the kernel
-# sources hash to the value they had at capture time.
+# DRAM bytes (read + write) of the seed search's kernel per read from one ncu
+# capture (a few hundred thousand reads, scaled per read; the profile summaries under
+# profiles/ give the command).  Used only while the kernel sources hash to the value
+# they had at capture time.
 KERNEL_SOURCES = ("aln_device.cuh", "aln_search.cuh", "aln_seed.cuh", "aln_flat.cuh", "aln_kernels.cu")
-TRAFFIC_CAPTURE = {  # workload -> capture; the profile summaries give the commands
+TRAFFIC_CAPTURE = {  # workload -> capture.  None of the 3.1 Gbp ones: they hold 51 GB, too much to profile on a shared GPU
     # 300 000 of the 1 M reads, aln_seed_kernel: 897.7 MB read + 34.1 MB written
     "chr100": {"src_sha256_16": "dba846bc96dc139f", "dram_bytes_per_read": 3106},
-    # 300 000 mates of the same recipe, aln_seed_kernel and aln_seed_wide_kernel:
-    # 1808.0 + 67.4 MB and 928.9 + 6.8 MB
-    "human_pairs": {"src_sha256_16": "dba846bc96dc139f", "dram_bytes_per_read": 9370},
 }
 L2_BYTES = 126 << 20  # GB300 L2 (cudaDevAttrL2CacheSize reports 126 MiB)
 
