@@ -430,22 +430,22 @@ def workload_config(name, w, n_per_step, ws, mode="persistent"):
             "parallelism": f"replicas{ws}" if ws > 1 else "single"}
 
 
-def search_launches(aln, params, scratch=True):
-    """Kernels one search of more than 2048 reads launches (the same list whether
-    launched directly or replayed from a graph): the plain form one; the persistent
-    form the tree search, with scratch three before it (the seed search, its wide
-    form and the D scan of the rest; of limits it does not take, the D pre-pass and
-    the two visit-order kernels), and unless the heavy phase is off its start kernel
-    and one pass and one decide kernel per deepening pass after it (one kernel in
-    all for a seed search of at most 2048 reads)."""
+def search_launches(aln, params, scratch=True, n_reads=None):
+    """Kernels one search launches on an index with its derived arrays (the same list
+    whether launched directly or replayed from a graph): the plain form one; the
+    persistent form the tree search, with scratch three before it (the seed search,
+    its wide form and the D scan of the rest; of limits it does not take, the D
+    pre-pass and the two visit-order kernels), and unless the heavy phase is off its
+    start kernel and one pass and one decide kernel per deepening pass after it, or
+    one kernel in all for a seed search of at most 2048 reads (n_reads; None: more)."""
     if params.mode == aln.MODE_PLAIN:
         return 1
-    n = 1
-    if scratch:
-        n += 3
-        if params.heavy_after != 0xFFFFFFFF:
-            n += 1 + 2 * aln.HEAVY_PASSES
-    return n
+    if not scratch:
+        return 1
+    seeded = min(params.max_gapo, params.z) <= 1 and not params.work_limit and not params.loop_limit
+    if params.heavy_after == 0xFFFFFFFF:
+        return 4
+    return 4 + (1 if seeded and n_reads is not None and n_reads <= 2048 else 1 + 2 * aln.HEAVY_PASSES)
 
 
 def time_search(al, d, params, res, hits, stream, flush, steps, warmup, torch, graph=None):
@@ -602,7 +602,7 @@ def human_phase(args, aln, torch, dev, stream, flush):
                       "bit_identical_to_persistent_on_complete_reads": same}
         b["persistent_over_plain"] = ms_l / ms_p
         b["flags"] = _flag_counts(aln, rq)
-        b["gpu_launches_per_step"] = {"persistent": search_launches(aln, pp), "plain": search_launches(aln, pl)}
+        b["gpu_launches_per_step"] = {"persistent": search_launches(aln, pp, n_reads=n), "plain": search_launches(aln, pl)}
         b["_out"] = (w, rq, hq, ms_p)
         blocks[name] = b
         del d, res, hits, graph
@@ -914,7 +914,7 @@ def run_gpu(args):
                      "reads_per_rank": [partition_range(n, r, ws)[1] - partition_range(n, r, ws)[0]
                                         for r in range(ws)]},
         # timed regions: the persistent steps and the plain steps (search_launches)
-        "gpu_launches": args.steps * (search_launches(aln, params["persistent"])
+        "gpu_launches": args.steps * (search_launches(aln, params["persistent"], n_reads=n_local)
                                       + search_launches(aln, params["plain"])),
         "e2e": {"value": e2e_v, "unit": "reads/s", "h2d_bytes_per_step": int(h2d) * ws,
                 "d2h_bytes_per_step": int(d2h) * ws, "hits_compacted": "aln_compact_hits",

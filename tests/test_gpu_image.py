@@ -78,3 +78,20 @@ def test_text_too_long_to_walk(torch):
         ok = npos == 1
         assert ok.any() and (npos[~ok] == aln.POS_WALK_LIMIT).all()
         assert np.array_equal(pos[ok, 0].astype(np.int64), (sa if strand else n - sa.astype(np.int64))[ok])
+
+
+def test_period_of_two_is_derived(torch):
+    """Its walks stay far below the bound, so every row has a position."""
+    text = np.tile(np.array([0, 3], np.uint8), 20_000)
+    ox = oracle.OracleIndex(text)
+    assert _longest_walk(ox.sa(0), 32) < 64 * 32
+    al = aln.Aligner(aln.Index.build(text).to_device(0))
+    assert al.dix.derived_bytes() > 0
+    n = text.size
+    hits = np.zeros(n + 1, aln.HIT_DTYPE)
+    hits["k"] = hits["l"] = np.arange(n + 1)
+    for strand, sa in ((1, ox.sa(0)), (0, ox.sa(1))):
+        hits["strand"] = strand
+        pos, npos = al.positions(hits, 1)
+        assert (npos == 1).all()
+        assert np.array_equal(pos[:, 0].astype(np.int64), sa.astype(np.int64) if strand else n - sa.astype(np.int64))
