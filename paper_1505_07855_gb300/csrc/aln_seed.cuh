@@ -758,8 +758,12 @@ __device__ SeedAnswer seed_search(const DIndex &X, const ReadBatch &rb, const Se
             todo = false;
         }
         const uint32_t span = ps | (pe << 8) | (off << 16);
-        for (uint32_t c0 = 0; __any_sync(FULL, todo && c0 < total); c0 += G) {
-            const uint32_t c = c0 + l, have = min(S.count, static_cast<uint32_t>(E));
+        // A group that has found more targets than it keeps is done: of a family of
+        // thousands of similar copies it would look at every place for nothing (50 000
+        // reads of 20 bases out of 5000 copies 1 % apart: the wide kernel 247 ms, now 10;
+        // 20 000 of 36 bases at z = 3: 223 ms, now 30).
+        for (uint32_t c0 = 0; __any_sync(FULL, todo && c0 < total && S.count <= static_cast<uint32_t>(E)); c0 += G) {
+            const uint32_t c = c0 + l, found = S.count, have = min(found, static_cast<uint32_t>(E));
             __syncwarp();  // before lanes record targets
             uint32_t o = 0;  // the lane whose part has place c: the last one that starts at or before it
 #pragma unroll
@@ -772,7 +776,7 @@ __device__ SeedAnswer seed_search(const DIndex &X, const ReadBatch &rb, const Se
             const uint32_t ospan = __shfl_sync(FULL, span, static_cast<int>(o), G);
             const uint32_t cs = o / kHalf;
             const int qs = static_cast<int>(ospan & 0xFFu), qe = static_cast<int>((ospan >> 8) & 0xFFu);
-            bool live = todo && c < total;
+            bool live = todo && c < total && found <= static_cast<uint32_t>(E);
             long long d = 0;  // the diagonal: text position of pattern index 0
             if (live) {
                 d = static_cast<long long>(__ldg(X.sa[0] + orow)) - static_cast<int>(ospan >> 16);
