@@ -377,7 +377,10 @@ struct FlatLane {
 #endif
             if (phase == PH_IDLE) {
                 if (heavy_seen) return;  // stay idle this trip: the hand-over may give it a heavy read's subtree
-                r = atomicAdd(queue, 1u);
+                // a helper that comes back asks first, or its lanes would carry the
+                // counter past its range
+                r = *reinterpret_cast<volatile uint32_t *>(queue);
+                if (r < n_reads) r = atomicAdd(queue, 1u);
                 if (r >= n_reads) {
                     phase = PH_FREE;
                     return;
