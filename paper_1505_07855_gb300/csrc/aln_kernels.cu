@@ -318,10 +318,10 @@ __device__ void heavy_start_one(const HeavyCtx &H, uint32_t hid, const uint2 *db
 }
 
 // Blocks of the start and decide kernels per SM: a call without heavy reads, the
-// usual one, only pays for launching them (1.3 us with 1 block an SM, 1.4 with 4,
-// 2.1 with one a possible read, 2048), and clearing the tables of 2048 heavy reads
-// takes 41, 20 and 15 us.
-constexpr uint32_t kHeavyBlocksPerSm = 4;
+// usual one, only pays for launching them (1.3 us with 1 or 2 blocks an SM, 1.4 with
+// 4, 2.1 with one a possible read, 2048); clearing the tables of 2048 heavy reads
+// takes 41 / 25 / 20 / 15 us, writing their results 110 us with 2, 90 with 4.
+constexpr uint32_t kHeavyBlocksPerSm = 2;
 
 __global__ void aln_heavy_start_kernel(SearchParams p, const uint2 *dbp, uint32_t n_text) {
     cudaGridDependencySynchronize();
@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_heavy
 // it.  A thread places a hit by the number of listed hits before it, so a read of
 // n listed hits takes n / 128 rounds over them.  (One thread, searching the 2048
 // slots for each hit in turn, took 8.9 ms for 2048 reads, a block each, and 11.4 ms
-// on 152 blocks; this takes 0.09 ms on 608.)
+// on 152 blocks; this takes 0.11 ms on 304.)
 __device__ void heavy_write(const SearchParams &p, const HeavySlot *T, const HeavyRead *R, uint32_t fin,
                             aln_read_result *res, aln_hit *hits) {
     constexpr uint32_t kSlots = 2 * kHeavySlots;
