@@ -548,9 +548,11 @@ extern "C" int aln_pack_reads(const uint8_t *codes, const uint64_t *code_offset,
     }
     if (total == 0) return ALN_OK;
     // ranges of reads, one a thread (a range of 2^18 bases takes about 0.1 ms on
-    // one core); a range's first and last words may be shared with its neighbours
-    const uint64_t most = std::min<uint64_t>(16, static_cast<uint64_t>(resolve_threads(0)));
-    const uint64_t ranges = std::max<uint64_t>(1, std::min<uint64_t>({most, total >> 18, n_reads}));
+    // one core); a range's first and last words may be shared with its neighbours.
+    // The number of cores costs more to ask for than a small batch to pack (one read:
+    // 30 us with the question, 15 without).
+    uint64_t ranges = std::min<uint64_t>({16, total >> 18, n_reads});
+    ranges = ranges < 2 ? 1 : std::min<uint64_t>(ranges, static_cast<uint64_t>(resolve_threads(0)));
     auto first_read = [&](uint64_t i) { return static_cast<uint32_t>(n_reads * i / ranges); };
     for (uint64_t i = 0; i <= ranges; i++) {
         const uint64_t at = i < ranges ? std::min(offset_out[first_read(i)], total - 1) : total - 1;
