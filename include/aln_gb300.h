@@ -80,8 +80,8 @@ extern "C" {
 #define ALN_STATUS_LOOP_LIMIT 0x1u   /* a warp of the persistent launch reached params.loop_limit */
 
 /* ---------------------------------------------------------------- modes */
-#define ALN_MODE_PLAIN 0      /* one launch per batch, one thread per read */
-#define ALN_MODE_PERSISTENT 1 /* one persistent launch; threads pull reads from a device queue */
+#define ALN_MODE_PLAIN 0      /* one launch per batch; trees searched one thread per read */
+#define ALN_MODE_PERSISTENT 1 /* a persistent tree search: threads pull reads from a device queue */
 #define ALN_STRATA_BEST1 0    /* keep hits with diffs <= min(z, d_best + 1) */
 #define ALN_STRATA_FULL 1     /* keep every hit with diffs <= z */
 #define ALN_STRATA_SCORE 2    /* score-ordered (persistent form only): every hit within z with

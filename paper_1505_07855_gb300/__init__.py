@@ -275,9 +275,10 @@ class Aligner:
         """Capture one search of the uploaded batch d into a CUDA graph; replay it
         with graph.replay() for every new batch copied into the same buffers.
         The graph owns a queue counter of its own and a scratch buffer (kept on
-        the graph object as ``aln_scratch``) for the D pre-pass and visit order,
-        so a replay runs the same four kernels as aln_search.  Replays of one
-        graph must not overlap each other."""
+        the graph object as ``aln_scratch``) for the lists of the seed search or the
+        D pre-pass and visit order, and for the heavy phase, so a replay runs the
+        kernels that aln_search runs.  Replays of one graph must not overlap each
+        other."""
         t = self.torch
         scratch = t.empty(scratch_bytes(d["n"]), dtype=t.uint8, device=self.dev)
         side = t.cuda.Stream(device=self.dev)

@@ -1,9 +1,11 @@
 // Search kernels and their launcher.
 //
-// Plain form: one launch per batch, one thread per read (both strands).
-// Persistent form: one launch of (SMs x resident blocks); every thread pulls the
-// next read from a device queue counter when it finishes one, so a few long
-// reads no longer hold a whole warp's worth of short ones.
+// Both forms answer most reads from seeds (aln_seed.cuh) and search the trees of the
+// others.  Plain form: one launch per batch, in which a warp looks up the seeds of its
+// reads and then searches one tree a lane.  Persistent form: the seed search, a wider
+// one, the D scan of the reads left, and one launch of (SMs x resident blocks) in which
+// a lane pulls its next read from a device queue counter, so a few long reads do not
+// hold a whole warp's worth of short ones; then the heavy phase.
 //
 // Stack bound: the match child is pushed below the alternatives, so entries on
 // the stack have non-decreasing difference counts from bottom to top and a
@@ -74,7 +76,8 @@ __global__ void __launch_bounds__(kThreads) aln_plain_kernel(DIndex X, ReadBatch
 // tree search alone takes 66.6 and 24.0; 100 000 reads of 100 bases on 100 Mbp, next
 // to none of them left, 0.455 ms (0.475, and 52).  Resident blocks an SM: 5 / 6 / 7 /
 // 8 take 76.5 / 70.6 / 69.2 / 70.2 and 27.8 / 23.1 / 25.9 / 27.7 ms for the copies,
-// 0.571 / 0.455 / 0.452 / 0.434 for the others.
+// 0.571 / 0.455 / 0.452 / 0.434 for the others.  (With the gapped stage in line as it
+// is now, 71.2, 22.4 and 0.415 ms with 6.)
 #ifndef ALN_PLAIN_BLOCKS
 #define ALN_PLAIN_BLOCKS 6
 #endif
@@ -94,7 +97,7 @@ __global__ void __launch_bounds__(kThreads, kPlainBlocks) aln_plain_seed_kernel(
     for (uint32_t t = 0; t < warp_reads && first + t < n_reads; t += kPlainStep) {
         const uint64_t r = first + t + group % kPlainStep;
         const bool active = t + group % kPlainStep < warp_reads && r < n_reads;
-        const SeedAnswer got = seed_search<kPlainLanes, kPlainTargets, false, true>(
+        const SeedAnswer got = seed_search<kPlainLanes, kPlainTargets, false>(
             X, rb, p, s_read[group], static_cast<uint32_t>(r), active, kPlainPlaces, res, hits);
         const bool rest = active && got != kSeedDone && threadIdx.x % kPlainLanes == 0;
         const unsigned all = __ballot_sync(0xFFFFFFFFu, rest);
@@ -734,8 +737,8 @@ __global__ void aln_heavy_decide_kernel(SearchParams p, const uint2 *dbp, uint32
 
 // The whole phase in one cooperative launch, a grid barrier where the kernels
 // above follow each other: for a call of at most kHeavyReads reads, whose time is
-// that of its launches when, as usual, no read is heavy (a call of 64 reads
-// launched 11 kernels to find that out).
+// that of its launches when, as usual, no read is heavy (64 reads take 29 us so, 47
+// with the eleven kernels).
 template <int STACK_CAP, bool SCORE>
 __global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_heavy_all_kernel(
     DIndex X, ReadBatch rb, SearchParams p, const uint2 *dbp, aln_read_result *res, aln_hit *hits) {
@@ -813,7 +816,7 @@ struct SeedCounts {          // in the scratch's first words, cleared before the
 
 // Room for targets and places to look at, first for a read's 8 or 16 lanes: past
 // that the other reads of the warp wait for it, so it goes to a warp of its own
-// (300 000 mates on 3.1 Gbp: 8.4 / 7.15 / 6.2 ms with 1024 / 256 / 64 places).
+// (300 000 mates on 3.1 Gbp: 6.96 / 5.91 / 5.36 ms with 1024 / 256 / 64 places).
 // There, kCandCap targets are what the tree search keeps.
 constexpr uint32_t kSeedTargets = 32;
 #ifndef ALN_SEED_PLACES
@@ -821,8 +824,8 @@ constexpr uint32_t kSeedTargets = 32;
 #endif
 constexpr uint32_t kSeedPlaces = ALN_SEED_PLACES;
 
-// Resident blocks per SM: 4 / 5 / 6 take 3.36 / 3.08 / 2.98 ms for 1 M reads of 100
-// bases on 100 Mbp and 6.28 / 5.87 / 5.76 ms for 300 000 mates on 3.1 Gbp (latency; 6
+// Resident blocks per SM: 4 / 5 / 6 take 3.39 / 3.11 / 3.00 ms for 1 M reads of 100
+// bases on 100 Mbp and 5.85 / 5.48 / 5.36 ms for 300 000 mates on 3.1 Gbp (latency; 6
 // spills in the gapped path); the wide kernel is the same with 4 and 5.
 #ifndef ALN_SEED_MIN_BLOCKS
 #define ALN_SEED_MIN_BLOCKS 6
@@ -938,8 +941,8 @@ __global__ void aln_order_scatter_kernel(const uint2 *dbp, uint32_t n, const uin
 
 // A launch that may be prepared while the kernel before it on the stream drains
 // (the kernel waits for it at its start): most of a call's kernels find nothing
-// to do, and a call's time is then that of its launches (64 reads: 77 -> 58 us
-// with the heavy phase in one launch; 30 000 reads: 195 -> 162 us).
+// to do, and a call's time is then that of its launches.  64 reads take 35 us without
+// and 29 with it, 10 000 in a graph 49.6 and 45.1, 30 000 155 and 117.
 template <class... Params, class... Args>
 static cudaError_t launch_after(void (*kernel)(Params...), unsigned blocks, cudaStream_t st, const SearchParams *window,
                                 Args &&...args) {

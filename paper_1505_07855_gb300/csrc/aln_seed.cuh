@@ -28,7 +28,7 @@
 // the other, this takes 2 (z + 1) look-ups at once and looks at about ten places
 // (100 Mbp), each a read of the suffix array and of the text.  1 M reads of 100
 // bases at z = 4 on 100 Mbp: 65 -> 3.0 ms; 400 000 reads of 36 to 250 bases on
-// 3.1 Gbp: 738 -> 14.8 ms.  It is bound by the latency of
+// 3.1 Gbp: 738 -> 14.1 ms.  It is bound by the latency of
 // those four dependent random reads and by instruction issue, not by bandwidth.
 #pragma once
 
@@ -42,7 +42,7 @@ namespace aln {
 #define ALN_EXTEND 24
 #endif
 // Bases a part grows by at most, past the table's: 300 000 mates on 3.1 Gbp take
-// 8.03 / 7.54 / 7.28 ms with 6 / 12 / 24, unique reads do not grow at all.
+// 5.47 / 5.42 / 5.36 ms with 6 / 12 / 24, unique reads do not grow at all.
 constexpr int kExtend = ALN_EXTEND;
 constexpr uint32_t kWideRows = 1u << 20;  // a part's rows saturate here
 #ifndef ALN_MANY_PLACES
@@ -50,7 +50,7 @@ constexpr uint32_t kWideRows = 1u << 20;  // a part's rows saturate here
 #endif
 // Places per lane from which a pass starts over with fewer, longer parts.  1, 2, 3, 6
 // and 8 are within 2 % of each other on the 3.1 Gbp batches (1 costs unique reads
-// of 100 Mbp 12 %).
+// of 100 Mbp 13 %).
 constexpr uint32_t kManyPlaces = ALN_MANY_PLACES;
 
 // Row of the suffix of text w that starts at position pos (0 .. n).
@@ -386,13 +386,6 @@ __device__ __forceinline__ uint32_t gap_targets(const uint2 *text, uint32_t n, S
     return found;
 }
 
-template <int G, int E>
-__device__ __noinline__ uint32_t gap_targets_call(const uint2 *text, uint32_t n, SeedRead<E> &S, uint32_t have, int m,
-                                                  long long d, int first_end, int last_start, uint32_t F, uint32_t gmost,
-                                                  int e, SeedZone Z) {
-    return gap_targets<G, E>(text, n, S, have, m, d, first_end, last_start, F, gmost, e, Z);
-}
-
 // Bitonic sort of a read's first P entries (a power of two, the same for every
 // group of the warp) by its G lanes; less(i, j) compares two entries.
 template <int G, int E, class Less>
@@ -593,10 +586,10 @@ enum SeedAnswer : uint32_t { kSeedDone, kSeedWide, kSeedTree };
 constexpr uint32_t kWidePlaces = 16384;
 
 // Search of one read by the G lanes of a group; all 32 lanes of the warp call it
-// together (other groups with their own reads, or with active = false).  CALL: the gapped stage out of line
-// (1 M reads take 3.37 ms with it and 2.93 without; in the plain kernel, whose tree
-// search takes its registers, 100 000 take 0.48 ms with it and 1.25 without).
-template <int G, int E, bool SCORE, bool CALL = false>
+// together (other groups with their own reads, or with active = false).  The
+// gapped stage is in line: 1 M reads take 3.41 ms with it in a function of its own and
+// 3.00 without, 100 000 in the plain form 0.457 and 0.419.
+template <int G, int E, bool SCORE>
 __device__ SeedAnswer seed_search(const DIndex &X, const ReadBatch &rb, const SearchParams &p, SeedRead<E> &S, uint32_t r,
                             bool active, uint32_t max_places, aln_read_result *res, aln_hit *hits) {
     constexpr unsigned FULL = 0xFFFFFFFFu;
@@ -835,8 +828,7 @@ __device__ SeedAnswer seed_search(const DIndex &X, const ReadBatch &rb, const Se
                 const int ls = 255 - static_cast<int>(group_min<G>(same ? 255u - static_cast<uint32_t>(qs) : 255u));
                 if (left) {
                     const int e = static_cast<int>(p.e);
-                    dgap = min(dgap, CALL ? gap_targets_call<G, E>(X.text, n, S, have, m, dd, fe, ls, F, gmost, e, zone(ds))
-                                          : gap_targets<G, E>(X.text, n, S, have, m, dd, fe, ls, F, gmost, e, zone(ds)));
+                    dgap = min(dgap, gap_targets<G, E>(X.text, n, S, have, m, dd, fe, ls, F, gmost, e, zone(ds)));
                 }
                 left &= ~__ballot_sync(FULL, same);
             }
@@ -853,7 +845,7 @@ __device__ SeedAnswer seed_search(const DIndex &X, const ReadBatch &rb, const Se
             } else if (exhaustive || F <= b) {  // F = z while nothing is found
                 todo = false;
             } else {
-                b = stepping ? min(F, 2 * b + 1) : F;  // 1, 2, 3, ... takes the mixed batch 18.1 ms, this 14.8
+                b = stepping ? min(F, 2 * b + 1) : F;  // 1, 2, 3, ... takes 300 000 mates on 3.1 Gbp 5.78 ms, this 5.33
             }
         }
     }
