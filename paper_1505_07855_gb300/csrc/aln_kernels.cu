@@ -136,9 +136,11 @@ __global__ void __launch_bounds__(kThreads, ALN_PERSISTENT_MIN_BLOCKS) aln_persi
     // The reads that a seed search has left are few and heavy: they go to all warps
     // of the grid, and a warp's other lanes help from the start.  (Taken up 32 a warp,
     // 1284 of 50 000 reads of 60 bases out of 3000 copies 5 % apart took the first 41
-    // warps 353 ms, where the tree search of all of them takes 46; now 19.)
-    const uint32_t warps = gridDim.x * (kThreads / 32);
-    const bool takes = !left || static_cast<uint64_t>(lane) * warps < *left;
+    // warps 353 ms, where the tree search of all of them takes 46; now 19.  Where three
+    // quarters of the lanes would have a read, all take one: 100 000 reads of one letter
+    // 4.2 ms, 4.7 shared out.)
+    const uint64_t warps = static_cast<uint64_t>(gridDim.x) * (kThreads / 32);
+    const bool takes = !left || *left >= 24 * warps || lane * warps < *left;
     L.phase = takes ? PH_IDLE : PH_FREE;
     L.r = 0xFFFFFFFFu;
     L.sp = 0;
