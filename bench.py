@@ -39,8 +39,8 @@ BYTES_PER_LOOKUP = 64
 # they had at capture time.
 KERNEL_SOURCES = ("aln_device.cuh", "aln_search.cuh", "aln_seed.cuh", "aln_flat.cuh", "aln_kernels.cu")
 TRAFFIC_CAPTURE = {  # workload -> capture.  None of the 3.1 Gbp ones: they hold 51 GB, too much to profile on a shared GPU
-    # 300 000 of the 1 M reads, aln_seed_kernel: 897.7 MB read + 34.1 MB written
-    "chr100": {"src_sha256_16": "dba846bc96dc139f", "dram_bytes_per_read": 3106},
+    # 300 000 of the 1 M reads, aln_seed_kernel: 897.2 MB read + 34.4 MB written
+    "chr100": {"src_sha256_16": "086e3365368e68f1", "dram_bytes_per_read": 3105},
 }
 L2_BYTES = 126 << 20  # GB300 L2 (cudaDevAttrL2CacheSize reports 126 MiB)
 

@@ -130,9 +130,9 @@ int fm_index_info(const fm_index *idx, fm_index_info_t *info);
  * and errors are those of fm_index_build, and the result is the same host index,
  * byte for byte (the suffix array is unique; everything else is a function of
  * it).  device: CUDA ordinal that does the work; stream: the work is enqueued on
- * it and finished before return.  The call allocates about 45 * (n + 1) bytes of
+ * it and finished before return.  The call allocates about 47 * (n + 1) bytes of
  * device memory for its duration (suffix array by prefix doubling with radix
- * sorts of (u64, u32) pairs) and frees it before return; ALN_ENOMEM if that does
+ * sorts of up to (u64, u32) pairs) and frees it before return; ALN_ENOMEM if that does
  * not fit, ALN_EDEVICE on a CUDA failure. */
 int fm_index_build_gpu(const uint8_t *text, uint64_t n, const fm_build_opts *opts, int device, void *stream,
                        fm_index **out);
@@ -308,8 +308,9 @@ typedef struct {
  * lane are handed to the heavy phase (at most 2048 per call), which searches
  * them from the deepening pass they were in, one pass per launch, with every
  * lane of the GPU sharing their subtrees through a task ring; it adds
- * 1 + 2 * ALN_HEAVY_PASSES launches to every persistent call with scratch
- * (they return at once when no read was handed over).  Its scratch is out->scratch
+ * 1 + 2 * ALN_HEAVY_PASSES launches to every persistent call with scratch, or one
+ * to a call of at most 2048 reads that is first answered from seeds (they return
+ * at once when no read was handed over).  Its scratch is out->scratch
  * if given, else a block from a memory pool owned by the device index,
  * allocated and freed in stream order by the call.  While stream is being
  * captured into a graph without out->scratch (or if the pool cannot serve) the

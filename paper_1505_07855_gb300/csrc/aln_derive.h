@@ -13,7 +13,7 @@ struct DIndex;
 #define ALN_LO_STRINGS 4
 #endif
 // Strings in the k-mer table per suffix, at most: with 4 (14-mers at 100 Mbp, 1.1
-// GB) 1 M reads take 3.7 ms, with 1 (13-mers) 4.9 ms, as every part then has a
+// GB) 1 M reads take 3.0 ms, with 1 (13-mers) 4.1 ms, as every part then has a
 // chance place or two.
 constexpr uint64_t kLoStrings = ALN_LO_STRINGS;
 
